@@ -327,6 +327,17 @@ int learned_prepare(dvm_ctx *c)
     return rc ? fail(c, rc, "hard-sphere scratch allocation failed") : DVM_OK;
 }
 
+dvm::MomGrid mom_grid(const dvm_ctx *c)
+{
+    dvm::MomGrid g;
+    for (int d = 0; d < 3; d++) {
+        g.half[d] = c->half[d];
+        g.hv[d] = c->hv[d];
+    }
+    g.dV = c->dV;
+    return g;
+}
+
 dvm::StepParams collision_params(dvm_ctx *c, double *mom)
 {
     dvm::StepParams p{};
@@ -1287,7 +1298,7 @@ int dvm_moments(dvm_ctx *c, double *rho, double *u, double *T)
 {
     if (!c) return DVM_EINVAL;
     if (c->state < 3) return fail(c, DVM_ESTATE, "f is not set");
-    int rc = dvm::launch_moments(c->cfg.precision, c->d_f[c->cur], ncells_of(c), c->nv, c->d_xi, c->dV, c->d_mom2, c->stream);
+    int rc = dvm::launch_moments(c->cfg.precision, c->d_f[c->cur], ncells_of(c), mom_grid(c), c->d_mom2, c->stream);
     if (rc) return fail(c, rc, "moments launch failed");
     return copy_moments(c, c->d_mom2, rho, u, T);
 }
@@ -1319,7 +1330,7 @@ static int kn_local_device(dvm_ctx *c)
         if (rc) return rc;
         c->ks_cells = nc;
     }
-    int rc = dvm::launch_moments(c->cfg.precision, c->d_f[c->cur], nc, c->nv, c->d_xi, c->dV, c->d_mom2, c->stream);
+    int rc = dvm::launch_moments(c->cfg.precision, c->d_f[c->cur], nc, mom_grid(c), c->d_mom2, c->stream);
     if (!rc) rc = dvm::launch_kn_local(c->d_mom2, c->d_ks_start, c->d_ks_nb, c->d_ks_coef, nc, c->cfg.kn, c->d_ks_knl, c->stream);
     return rc ? fail(c, rc, "Knudsen sensor launch") : DVM_OK;
 }
@@ -1442,7 +1453,7 @@ int dvm_hs_collide_noalloc(dvm_ctx *c, float *f, int64_t ncells, double dt)
     p.P = c->P;
     p.status = c->d_status;
     p.stream = c->stream;
-    int rc = dvm::launch_hs_collide_noalloc(c->hs, p, f, c->d_xi, c->dV, c->cfg.kn, dt);
+    int rc = dvm::launch_hs_collide_noalloc(c->hs, p, f, mom_grid(c), c->cfg.kn, dt);
     if (rc) return fail(c, rc, rc == DVM_EINVAL ? "scratch too small" : "hard-sphere launch failed");
     int st = 0;
     rc = cuda_check(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "read status");
@@ -1609,7 +1620,7 @@ int dvm_learned_collide(dvm_ctx *c, double dt, const float *o_in, double *knl, f
     if (rc) return rc;
     const int64_t nc = ncells_of(c);
     float *f = static_cast<float *>(c->d_f[c->cur]);
-    rc = dvm::launch_moments(DVM_F32, f, nc, c->nv, c->d_xi, c->dV, c->d_mom2, c->stream);
+    rc = dvm::launch_moments(DVM_F32, f, nc, mom_grid(c), c->d_mom2, c->stream);
     if (rc) return fail(c, rc, "moments launch failed");
     if (o_in) rc = cuda_check(c, cudaMemcpyAsync(c->d_lo, o_in, (size_t)nc * 256, cudaMemcpyHostToDevice, c->stream), "copy o");
     if (!rc && o_in && a)
@@ -1647,7 +1658,7 @@ int dvm_learned_pairs(dvm_ctx *c, float *a, float *o)
     DevArr dq(c, (size_t)nc * c->nv * 4), da(c, (size_t)nc * 256), dout(c, (size_t)nc * 256);
     if (!dq.p || !da.p || !dout.p) return fail(c, DVM_ENOMEM, "device allocation (training pairs)");
     float *f = static_cast<float *>(c->d_f[c->cur]);
-    rc = dvm::launch_moments(DVM_F32, f, nc, c->nv, c->d_xi, c->dV, c->d_mom2, c->stream);
+    rc = dvm::launch_moments(DVM_F32, f, nc, mom_grid(c), c->d_mom2, c->stream);
     if (!rc) rc = dvm::launch_hermite_project(f, c->d_mom2, c->d_amag, nc, c->n, c->dV, 0, nullptr, nullptr, da.f(),
                                               nullptr, c->d_status, c->stream);
     dvm::StepParams p = collision_params(c, c->d_mom2);

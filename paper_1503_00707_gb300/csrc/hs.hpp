@@ -64,10 +64,8 @@ int launch_hs_general(HsTables &t, const StepParams &p, float *f, const int32_t 
 
 // The same update on caller-owned f with a fixed, statically allocated
 // device scratch (no allocation).  Needs p.ncells * (8 nv + 40) bytes of
-// scratch at most DVM_HS_NOALLOC_SCRATCH_BYTES (else DVM_EINVAL); xi is the
-// node table [nv][3] in FP64 and dV the velocity cell volume.
-int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const double *xi, double dV,
-                              double kn, double dt);
+// scratch at most DVM_HS_NOALLOC_SCRATCH_BYTES (else DVM_EINVAL).
+int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const MomGrid &g, double kn, double dt);
 
 // Trials per node that the register-resident table layout supports.
 bool hs_trials_supported(int trials);

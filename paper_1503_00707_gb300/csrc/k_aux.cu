@@ -6,6 +6,7 @@
 #include "../../include/dvm.h"
 #include "common.cuh"
 #include "kernels.hpp"
+#include "quads.cuh"
 
 namespace dvm {
 
@@ -48,38 +49,248 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
     }
 }
 
-template <typename TS>
-__global__ void k_moments(const TS *f, int64_t ncells, int nv, const double *xi, double dV, double *out)
+// Moments of a stored f: rho, u, T of every cell in FP64, one CTA per cell.
+//
+// A value enters only through the seven integer-weighted sums sum f,
+// sum j_d f, sum j_d^2 f (xi_d = (h_d/2) j_d, j_d odd).  FP64 runs at 1/64 of
+// the FP32 rate here and thirteen FP64 operations a value bound the kernel at
+// 57 GB/s of its read of f, so FP32 and BF16 storage sum exactly in fixed
+// point instead: with M the cell's largest |f| and sigma = 2^k >= 512 M, each
+// value splits without error (the extraction of Rump, Ogita and Oishi, 2008)
+// into a multiple of 2^(k-24), a multiple of 2^(k-39) and a rest of at most
+// 2^(k-39).  A thread's sums of its 32 values of either multiple, with the
+// weights that k_step's partials use (total size below 16 against the split's
+// margin), are exact in FP32 and go into 64-bit integers; the rests are summed
+// in FP32.  What is lost is below 2^-60 of sum |f|, less than FP64 summation
+// loses.  f is read once from HBM: a thread keeps its first two quads of
+// positions (32 values each) in registers between the search for M and the
+// sums; positions beyond that (grids of more than 512 quads) are read again.
+// A cell with non-finite values or M outside [2^-86, 2^115] takes FP64 sums.
+// 17,680 cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 319 us now
+// (3.1 TB/s, the registers of two quads a thread hold two CTAs an SM).
+constexpr int MOM_T = 256, MOM_HOLD = 2;
+
+__device__ inline uint32_t abs_bits(float2 v) { return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu); }
+
+// the seven base sums of a quad at one level of the split, times 2^-quantum
+// as integers: S, X, Y, Z over the four positions, sum e Z_e, sum e S_e,
+// sum e^2 S_e (e = 0..3)
+__device__ inline void base_sums(const float2 (&a)[8], const float2 (&b)[8], float (&s)[7])
 {
-    __shared__ double red[5][32];
-    const int64_t c = blockIdx.x;
-    double s[5] = {0, 0, 0, 0, 0};
-    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-        const double fv = to_double<TS>(f[c * nv + v]);
-        const double x = xi[3 * v], y = xi[3 * v + 1], z = xi[3 * v + 2];
-        s[0] += fv;
-        s[1] += x * fv;
-        s[2] += y * fv;
-        s[3] += z * fv;
-        s[4] += (x * x + y * y + z * z) * fv;
+    float2 Sa, Xa, Ya, Za, Sb, Xb, Yb, Zb;
+    group_sums(a, Sa, Xa, Ya, Za);
+    group_sums(b, Sb, Xb, Yb, Zb);
+    s[0] = (Sa.x + Sa.y) + (Sb.x + Sb.y);
+    s[1] = (Xa.x + Xa.y) + (Xb.x + Xb.y);
+    s[2] = (Ya.x + Ya.y) + (Yb.x + Yb.y);
+    s[3] = (Za.x + Za.y) + (Zb.x + Zb.y);
+    s[4] = (Za.y + 2.0f * Zb.x) + 3.0f * Zb.y;
+    s[5] = (Sa.y + 2.0f * Sb.x) + 3.0f * Sb.y;
+    s[6] = (Sa.y + 4.0f * Sb.x) + 9.0f * Sb.y;
+}
+
+// the seven weighted sums from the base sums (j = j0 + 2 e along z)
+template <typename T, typename J> __device__ inline void weighted_sums(const T (&s)[7], J jx, J jy, J jz, T (&m)[7])
+{
+    m[0] += s[0];
+    m[1] += s[1] * jx;
+    m[2] += s[2] * jy;
+    m[3] += s[3] * jz + s[4] * (J)2;
+    m[4] += s[0] * (jx * jx);
+    m[5] += s[0] * (jy * jy);
+    m[6] += s[0] * (jz * jz) + s[5] * (J)(4 * jz) + s[6] * (J)4;
+}
+
+// split a thread's 32 values at one level: x = q + r, q a multiple of
+// sigma 2^-24
+__device__ inline void extract8(float2 (&x)[8], float sigma, float2 (&q)[8])
+{
+    const float2 s2 = make_float2(sigma, sigma);
+#pragma unroll
+    for (int o = 0; o < 8; o++) {
+        q[o] = f2_sub(f2_add(x[o], s2), s2);
+        x[o] = f2_sub(x[o], q[o]);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < 5; k++) {
-        s[k] = warp_allsum(s[k]);
-        if (lane == 0) red[k][warp] = s[k];
+}
+
+struct MomSum {
+    int64_t I[7];  // in units of 2^(k-39)
+    float R[7];
+};
+
+__device__ inline void add_quad(const QV<float> (&x)[8], int ex, int jx, int jy, int jz, MomSum &m)
+{
+    const float sg1 = __int_as_float((ex + 10) << 23), sg2 = __int_as_float((ex - 5) << 23);  // 2^k, 2^(k-15)
+    const float c1 = __int_as_float((268 - ex) << 23), c2 = __int_as_float((283 - ex) << 23);  // 2^(24-k), 2^(39-k)
+    float2 ra[8], rb[8], qa[8], qb[8];
+#pragma unroll
+    for (int o = 0; o < 8; o++) {
+        ra[o] = x[o].a;
+        rb[o] = x[o].b;
+    }
+    float s1[7], s2[7], s3[7];
+    extract8(ra, sg1, qa);
+    extract8(rb, sg1, qb);
+    base_sums(qa, qb, s1);
+    extract8(ra, sg2, qa);
+    extract8(rb, sg2, qb);
+    base_sums(qa, qb, s2);
+    base_sums(ra, rb, s3);
+    int64_t v[7];
+#pragma unroll
+    for (int k = 0; k < 7; k++)
+        v[k] = (int64_t)__float2int_rn(s1[k] * c1) * 32768 + (int64_t)__float2int_rn(s2[k] * c2);
+    weighted_sums<int64_t, int>(v, jx, jy, jz, m.I);
+    weighted_sums<float, float>(s3, (float)jx, (float)jy, (float)jz, m.R);
+}
+
+// the same sums in FP64
+template <typename TC> __device__ inline void add_quad_f64(const QV<TC> (&x)[8], int jx, int jy, int jz, double (&m)[7])
+{
+    constexpr int VEC = sizeof(TC) == 8 ? 2 : 4;
+    double s[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+    for (int e = 0; e < VEC; e++) {
+        double S = 0, X = 0, Y = 0, Z = 0;
+#pragma unroll
+        for (int o = 0; o < 8; o++) {
+            double v;
+            if constexpr (sizeof(TC) == 8) v = e ? x[o].b : x[o].a;
+            else v = (double)(e == 0 ? x[o].a.x : e == 1 ? x[o].a.y : e == 2 ? x[o].b.x : x[o].b.y);
+            S += v;
+            X += (o & 4) ? v : -v;
+            Y += (o & 2) ? v : -v;
+            Z += (o & 1) ? v : -v;
+        }
+        s[0] += S;
+        s[1] += X;
+        s[2] += Y;
+        s[3] += Z;
+        s[4] += e * Z;
+        s[5] += e * S;
+        s[6] += e * e * S;
+    }
+    weighted_sums<double, double>(s, (double)jx, (double)jy, (double)jz, m);
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(MOM_T, 2)
+    k_moments(const TS *__restrict__ f, int P, int3 half, double3 hh, double dV, double *__restrict__ out)
+{
+    using IO = QIO<TS>;
+    using TC = typename Store<TS>::TC;
+    constexpr int VEC = Store<TS>::VEC;
+    __shared__ uint32_t wmax[MOM_T / 32];
+    __shared__ double red[MOM_T / 32][7];
+    __shared__ int64_t redI[MOM_T / 32][7];
+    __shared__ float redR[MOM_T / 32][7];
+    const int64_t c = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, nw = T >> 5, Q = P / VEC;
+    const TS *fc = f + c * 8 * (int64_t)P;
+    auto load = [&](int q, QV<TC> (&x)[8]) {
+#pragma unroll
+        for (int o = 0; o < 8; o++) x[o] = IO::ldg(fc + (int64_t)o * P + q * VEC);
+    };
+    auto nodes = [&](int q, int &jx, int &jy, int &jz) {
+        const int p = q * VEC, t = p / half.z;
+        jz = 2 * (p - t * half.z) + 1;
+        jy = 2 * (t % half.y) + 1;
+        jx = 2 * (t / half.y) + 1;
+    };
+    int jx, jy, jz;
+    bool wide = true;  // FP64 sums
+    int ex = 0;
+    if constexpr (sizeof(TC) == 4) {
+        QV<float> x[MOM_HOLD][8];
+        uint32_t mx = 0;
+        auto top = [&](const QV<float> (&v)[8]) {
+#pragma unroll
+            for (int o = 0; o < 8; o++) mx = max(mx, max(abs_bits(v[o].a), abs_bits(v[o].b)));
+        };
+#pragma unroll
+        for (int h = 0; h < MOM_HOLD; h++)
+            if (tid + h * T < Q) load(tid + h * T, x[h]);
+#pragma unroll
+        for (int h = 0; h < MOM_HOLD; h++)
+            if (tid + h * T < Q) top(x[h]);
+        for (int q = tid + MOM_HOLD * T; q < Q; q += T) {
+            QV<float> y[8];
+            load(q, y);
+            top(y);
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) wmax[warp] = mx;
+        __syncthreads();
+        for (int w = 0; w < nw; w++) mx = max(mx, wmax[w]);
+        ex = (int)(mx >> 23);  // M < 2^(ex - 126)
+        wide = ex < 40 || ex > 240;
+        if (!wide) {
+            MomSum m{};
+#pragma unroll
+            for (int h = 0; h < MOM_HOLD; h++)
+                if (tid + h * T < Q) {
+                    nodes(tid + h * T, jx, jy, jz);
+                    add_quad(x[h], ex, jx, jy, jz, m);
+                }
+#pragma unroll 1
+            for (int q = tid + MOM_HOLD * T; q < Q; q += T) {
+                QV<float> y[8];
+                load(q, y);
+                nodes(q, jx, jy, jz);
+                add_quad(y, ex, jx, jy, jz, m);
+            }
+            const int64_t I = warp_reduce7<int64_t>(m.I, lane);
+            const float R = warp_reduce7<float>(m.R, lane);
+            if ((lane & 3) == 0 && lane < 28) {
+                redI[warp][lane >> 2] = I;
+                redR[warp][lane >> 2] = R;
+            }
+        }
+    }
+    if (wide) {
+        double m[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+        for (int q = tid; q < Q; q += T) {
+            QV<TC> y[8];
+            load(q, y);
+            nodes(q, jx, jy, jz);
+            add_quad_f64<TC>(y, jx, jy, jz, m);
+        }
+        const double t = warp_reduce7<double>(m, lane);
+        if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
     }
     __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int k = 0; k < 5; k++) s[k] = warp_allsum(lane < nw ? red[k][lane] : 0.0);
-        if (lane == 0) {
-            const double s0 = s[0];
-            const double ux = s[1] / s0, uy = s[2] / s0, uz = s[3] / s0;
-            double *o = out + c * 5;
-            o[0] = s0 * dV;
-            o[1] = ux; o[2] = uy; o[3] = uz;
-            o[4] = (s[4] / s0 - (ux * ux + uy * uy + uz * uz)) / 3.0;
+    if (warp) return;
+    double s = 0.0;
+    if (lane < 7) {
+        if (wide) {
+            for (int w = 0; w < nw; w++) s += red[w][lane];
+        } else {
+            int64_t I = 0;
+            float R = 0.0f;
+            for (int w = 0; w < nw; w++) {
+                I += redI[w][lane];
+                R += redR[w][lane];
+            }
+            s = (double)I * __longlong_as_double((long long)(1023 + ex - 156) << 52) + (double)R;  // 2^(k-39)
         }
+    }
+    // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
+    const double s0 = __shfl_sync(0xffffffffu, s, 0);
+    const int d = (lane + 2) % 3;
+    const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
+    const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
+    const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
+    const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
+                 uz2 = __shfl_sync(0xffffffffu, u2, 3);
+    const double ex2 = __shfl_sync(0xffffffffu, e2, 1), ey2 = __shfl_sync(0xffffffffu, e2, 2),
+                 ez2 = __shfl_sync(0xffffffffu, e2, 3);
+    double *o = out + c * 5;
+    if (lane == 0) {
+        o[0] = s0 * dV;
+        o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
+    } else if (lane < 4) {
+        o[lane] = v;
     }
 }
 
@@ -216,15 +427,21 @@ int launch_init_maxwellian(int prec, void *f, int64_t ncells, int nv, int nmix, 
     return last_status();
 }
 
-int launch_moments(int prec, const void *f, int64_t ncells, int nv, const double *xi, double dV,
-                   double *out, cudaStream_t s)
+int launch_moments(int prec, const void *f, int64_t ncells, const MomGrid &g, double *out, cudaStream_t s)
 {
     if (ncells <= 0) return DVM_OK;
+    const int P = g.half[0] * g.half[1] * g.half[2], Q = P / (prec == DVM_F64 ? 2 : 4);
+    // one quad a thread up to 256 quads, then two (24^3: 432 quads on 224 threads)
+    const int per = Q <= MOM_T ? Q : (Q + 1) / 2, t = std::min(MOM_T, (per + 31) / 32 * 32);
     const dim3 grid((unsigned)ncells);
+    const int3 half = make_int3(g.half[0], g.half[1], g.half[2]);
+    const double3 hh = make_double3(0.5 * g.hv[0], 0.5 * g.hv[1], 0.5 * g.hv[2]);
     switch (prec) {
-    case DVM_F64: k_moments<double><<<grid, 256, 0, s>>>((const double *)f, ncells, nv, xi, dV, out); break;
-    case DVM_F32: k_moments<float><<<grid, 256, 0, s>>>((const float *)f, ncells, nv, xi, dV, out); break;
-    case DVM_BF16: k_moments<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16 *)f, ncells, nv, xi, dV, out); break;
+    case DVM_F64: k_moments<double><<<grid, t, 0, s>>>((const double *)f, P, half, hh, g.dV, out); break;
+    case DVM_F32: k_moments<float><<<grid, t, 0, s>>>((const float *)f, P, half, hh, g.dV, out); break;
+    case DVM_BF16:
+        k_moments<__nv_bfloat16><<<grid, t, 0, s>>>((const __nv_bfloat16 *)f, P, half, hh, g.dV, out);
+        break;
     default: return DVM_EINVAL;
     }
     return last_status();

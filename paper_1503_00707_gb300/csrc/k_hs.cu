@@ -583,8 +583,7 @@ int noalloc_scratch(void **ptr)
 
 }  // namespace
 
-int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const double *xi, double dV,
-                              double kn, double dt)
+int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const MomGrid &g, double kn, double dt)
 {
     if (p.prec != DVM_F32) return DVM_ENOTIMPL;
     if (!t.ready || t.nv != p.nv) return DVM_ESTATE;
@@ -599,12 +598,12 @@ int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const 
     if (rc) return rc;
     float *bc = static_cast<float *>(base);
     double *mom = reinterpret_cast<double *>(static_cast<unsigned char *>(base) + need_bc);
-    rc = launch_moments(DVM_F32, f, p.ncells, p.nv, xi, dV, mom, p.stream);
+    rc = launch_moments(DVM_F32, f, p.ncells, g, mom, p.stream);
     if (rc) return rc;
     rc = bc_launch(L, t, f, reinterpret_cast<float2 *>(bc), p.ncells, p.nv, nullptr, nullptr, p.stream, p.status);
     if (rc) return rc;
     k_hs_corr<<<(unsigned)p.ncells, CT, 0, p.stream>>>(f, reinterpret_cast<const float2 *>(bc), t.d_xi, t.d_jpk,
-                                                      t.hh, dV, mom, p.nv, make_int3(t.half[0], t.half[1], t.half[2]),
+                                                      t.hh, g.dV, mom, p.nv, make_int3(t.half[0], t.half[1], t.half[2]),
                                                       (float)(dt / kn), nullptr, nullptr, nullptr, nullptr, p.status);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;

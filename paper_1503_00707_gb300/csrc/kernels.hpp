@@ -49,9 +49,15 @@ int launch_init_maxwellian(int prec, void *f, int64_t ncells, int nv, int nmix,
                            const double *w, const double *rho, const double *u,
                            const double *T, const double *xi, cudaStream_t s);
 
+// The velocity grid as the moments of a stored f need it.
+struct MomGrid {
+    int half[3];   // n[d] / 2
+    double hv[3];  // spacing per axis
+    double dV;
+};
+
 // Moments of the stored f in FP64: out [ncells][5] = rho, u[3], T
-int launch_moments(int prec, const void *f, int64_t ncells, int nv, const double *xi,
-                   double dV, double *out, cudaStream_t s);
+int launch_moments(int prec, const void *f, int64_t ncells, const MomGrid &g, double *out, cudaStream_t s);
 
 // Convert count elements between storage precision and FP64.
 int launch_to_f64(int prec, const void *src, double *dst, int64_t count, cudaStream_t s);

@@ -445,8 +445,8 @@ int dvm_rank_moments(dvm_rank *r, double *rho, double *u, double *T)
 {
     if (!r) return DVM_EINVAL;
     if (!r->f_set) return rfail(r, DVM_ESTATE, "f is not set");
-    int rc = dvm::launch_moments(r->cfg.precision, r->d_f[r->cur], r->nown, r->g.nv, r->d_xi, r->g.dV, r->d_mom2,
-                                 r->stream);
+    const dvm::MomGrid g{{r->g.half[0], r->g.half[1], r->g.half[2]}, {r->g.hv[0], r->g.hv[1], r->g.hv[2]}, r->g.dV};
+    int rc = dvm::launch_moments(r->cfg.precision, r->d_f[r->cur], r->nown, g, r->d_mom2, r->stream);
     if (rc) return rfail(r, rc, "moments launch failed");
     std::vector<double> h(5 * (size_t)r->nown);
     rc = check(r, cudaMemcpyAsync(h.data(), r->d_mom2, h.size() * 8, cudaMemcpyDeviceToHost, r->stream), "copy moments");
