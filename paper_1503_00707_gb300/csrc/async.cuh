@@ -39,6 +39,13 @@ __device__ inline void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint
                  : "memory");
 }
 
+__device__ inline void bulk_g2s_addr(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
 __device__ inline bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 {
     uint32_t ok;

@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstring>
 #include <thread>
+#include <type_traits>
 
 #include "../../include/dvm.h"
 
@@ -317,13 +318,285 @@ static void order_for_banks(const std::vector<uint32_t> &idx, const std::vector<
     }
 }
 
+// Packed trials for the gather kernel that works on pairs of cells (64-bit
+// shared-memory gathers).  Only trials that carry weight (about 60%) are kept,
+// once in the tables of the sums B (one gather each) and once in those of the
+// sums C (two gathers each).  A node with c of them takes t lanes of one warp,
+// t the smallest power of two with c / t + 2 slots or fewer than the kind's
+// limit; a CTA runs the slots of its longest lane plus one or two, rounded up
+// to eight, and nodes are sorted by (t, that number), so that all warps of a
+// CTA do the same work.  A 64-bit gather is served half a warp at a time from
+// 16 banks of 8 bytes: within a half every distinct index in the same bank
+// (index mod 16) costs one more wavefront.  Each half's trials are placed
+// greedily, slot by slot, where they add no wavefront, the rest wherever there
+// is room, and then by seeded local search: moves and swaps of a node's trials
+// between its slots, with l and m exchanged at will (f_l f_m is symmetric).
+// Holding the two sums apart is what makes this work: one or two gathers of a
+// slot can be kept free of conflicts far more often than three together
+// (gathered values per wavefront, of 32: 24 and 23 for the two kinds, 20 for
+// three gathers in one slot, 16^3 and 24^3 grids with 128 trials).
+namespace {
+
+struct HalfSlot {
+    // per gather and bank: the distinct indices of a half warp's slot and how
+    // many lanes take each
+    uint8_t cnt[2][16];
+    uint8_t mult[2][16][16];
+    uint16_t addr[2][16][16];
+    int wave, sq;
+    void add(const uint16_t *a2, int ng, int sgn)
+    {
+        for (int g = 0; g < ng; g++) {
+            const int a = a2[g], bk = a & 15;
+            int pos = 0;
+            while (pos < cnt[g][bk] && addr[g][bk][pos] != a) pos++;
+            if (sgn > 0) {
+                if (pos == cnt[g][bk]) {
+                    cnt[g][bk]++;
+                    addr[g][bk][pos] = (uint16_t)a;
+                    mult[g][bk][pos] = 0;
+                }
+                mult[g][bk][pos]++;
+            } else if (--mult[g][bk][pos] == 0) {
+                const int last = --cnt[g][bk];
+                addr[g][bk][pos] = addr[g][bk][last];
+                mult[g][bk][pos] = mult[g][bk][last];
+            }
+        }
+    }
+    void cost(int ng, int &w, int &q) const
+    {
+        w = q = 0;
+        for (int g = 0; g < ng; g++) {
+            int mx = 1;
+            for (int k = 0; k < 16; k++) {
+                mx = std::max(mx, (int)cnt[g][k]);
+                q += cnt[g][k] * cnt[g][k];
+            }
+            w += mx;
+        }
+    }
+    // distinct indices the trial would add to occupied banks
+    int added(const uint16_t *a2, int ng) const
+    {
+        int c = 0;
+        for (int g = 0; g < ng; g++) {
+            const int bk = a2[g] & 15;
+            int pos = 0;
+            while (pos < cnt[g][bk] && addr[g][bk][pos] != a2[g]) pos++;
+            if (pos == cnt[g][bk]) c += cnt[g][bk];
+        }
+        return c;
+    }
+};
+
+struct PackTrial {
+    uint16_t a[2];  // gamma, or l and m
+    float b;
+};
+
+// one warp: nodes[k] and its weighted trials tr[k] on lanes k t .. k t + t - 1;
+// R slots
+void pack_warp(const std::vector<int> &nodes, std::vector<std::vector<PackTrial>> &tr, int kind, int t, int R,
+               uint64_t seed, uint32_t *tab, uint32_t *lane_tab)
+{
+    const int kn = (int)nodes.size(), ng = kind + 1, HM = hs_slots(kind);
+    std::vector<int> at((size_t)32 * HM, -1);  // index into tr[lane / t], or -1
+    std::vector<HalfSlot> S((size_t)2 * HM);
+    for (auto &x : S) std::memset(x.cnt, 0, sizeof x.cnt);
+    auto half = [&](int lane, int e) -> HalfSlot & { return S[(size_t)(lane >> 4) * HM + e]; };
+    std::vector<std::vector<uint8_t>> used(kn);
+    std::vector<int> left(kn);
+    for (int k = 0; k < kn; k++) {
+        used[k].assign(tr[k].size(), 0);
+        left[k] = (int)tr[k].size();
+    }
+    for (int pass = 0; pass < 2; pass++)
+        for (int e = 0; e < R; e++)
+            for (int lane = 0; lane < kn * t; lane++) {
+                const int k = lane / t;
+                int &p = at[(size_t)lane * HM + e];
+                if (!left[k] || p >= 0) continue;
+                HalfSlot &h = half(lane, e);
+                int best = -1, bc = INT_MAX;
+                bool flip = false;
+                for (int q = 0; q < (int)tr[k].size() && bc > 0; q++) {
+                    if (used[k][q]) continue;
+                    const uint16_t x[2] = {tr[k][q].a[0], tr[k][q].a[1]}, y[2] = {x[1], x[0]};
+                    const int c = h.added(x, ng), cf = kind ? h.added(y, ng) : INT_MAX;
+                    if (std::min(c, cf) < bc) {
+                        bc = std::min(c, cf);
+                        best = q;
+                        flip = cf < c;
+                    }
+                }
+                if (pass == 0 && bc > 0) continue;
+                if (flip) std::swap(tr[k][best].a[0], tr[k][best].a[1]);
+                used[k][best] = 1;
+                left[k]--;
+                h.add(tr[k][best].a, ng, +1);
+                p = best;
+            }
+    for (auto &x : S) x.cost(ng, x.wave, x.sq);
+    long total = 0;
+    for (int k = 0; k < kn; k++) total += (long)tr[k].size();
+    uint64_t st = mix64(seed);
+    for (long it = 0; it < (kind ? 60 : 30) * total && R > 1; it++) {
+        st = mix64(st);
+        const int k = (int)(st % (uint64_t)kn);
+        const int e1 = (int)((st >> 16) % (uint64_t)R), e2 = (int)((st >> 32) % (uint64_t)R);
+        const int l1 = k * t + (int)((st >> 48) % (uint64_t)t), l2 = k * t + (int)((st >> 56) % (uint64_t)t);
+        int &p1 = at[(size_t)l1 * HM + e1], &p2 = at[(size_t)l2 * HM + e2];
+        HalfSlot &h1 = half(l1, e1), &h2 = half(l2, e2);
+        if (&h1 == &h2 || (p1 < 0 && p2 < 0)) continue;
+        if ((p1 < 0 && h2.wave == ng) || (p2 < 0 && h1.wave == ng)) continue;  // nothing to gain by a move
+        // the trials before, and after the exchange (l and m flipped at will)
+        PackTrial o1{}, o2{}, n1{}, n2{};
+        if (p1 >= 0) n1 = o1 = tr[k][p1];
+        if (p2 >= 0) n2 = o2 = tr[k][p2];
+        if (kind && (st >> 40) & 1) std::swap(n1.a[0], n1.a[1]);
+        if (kind && (st >> 41) & 1) std::swap(n2.a[0], n2.a[1]);
+        if (p1 >= 0) h1.add(o1.a, ng, -1);
+        if (p2 >= 0) h2.add(o2.a, ng, -1);
+        if (p2 >= 0) h1.add(n2.a, ng, +1);
+        if (p1 >= 0) h2.add(n1.a, ng, +1);
+        int w1, q1, w2, q2;
+        h1.cost(ng, w1, q1);
+        h2.cost(ng, w2, q2);
+        const int dw = w1 + w2 - h1.wave - h2.wave, dq = q1 + q2 - h1.sq - h2.sq;
+        if (dw < 0 || (dw == 0 && dq <= 0)) {
+            if (p1 >= 0) tr[k][p1] = n1;
+            if (p2 >= 0) tr[k][p2] = n2;
+            std::swap(p1, p2);
+            h1.wave = w1;
+            h1.sq = q1;
+            h2.wave = w2;
+            h2.sq = q2;
+        } else {
+            if (p2 >= 0) h1.add(n2.a, ng, -1);
+            if (p1 >= 0) h2.add(n1.a, ng, -1);
+            if (p1 >= 0) h1.add(o1.a, ng, +1);
+            if (p2 >= 0) h2.add(o2.a, ng, +1);
+        }
+    }
+    for (int e = 0; e < HM; e++)
+        for (int hf = 0; hf < 2; hf++) {
+            // a lane without a trial gathers where another lane of its half does
+            const PackTrial *ref = nullptr;
+            for (int lane = 16 * hf; lane < 16 * hf + 16 && !ref; lane++)
+                if (at[(size_t)lane * HM + e] >= 0) ref = &tr[lane / t][at[(size_t)lane * HM + e]];
+            for (int lane = 16 * hf; lane < 16 * hf + 16; lane++) {
+                const int p = at[(size_t)lane * HM + e];
+                const PackTrial *x = p >= 0 ? &tr[lane / t][p] : ref;
+                const uint32_t a0 = x ? x->a[0] : 0u, a1 = x ? x->a[1] : 0u;
+                if (kind) tab[32 * e + lane] = (a0 << 3) | (a1 << 17);
+                else if (e & 1) tab[32 * (e / 2) + lane] |= a0 << 17;
+                else tab[32 * (e / 2) + lane] = a0 << 3;
+                const float b = p >= 0 ? x->b : 0.0f;
+                std::memcpy(&tab[32 * (HS_ROWS - HM + e) + lane], &b, 4);
+            }
+        }
+    int lg = 0;
+    while ((1 << lg) < t) lg++;
+    for (int lane = 0; lane < 32; lane++)
+        lane_tab[lane] = (lane / t < kn ? (uint32_t)nodes[lane / t] : HS_NO_NODE) | ((uint32_t)lg << 20);
+}
+
+}  // namespace
+
+void hs_pack(const std::vector<uint32_t> &idx, const std::vector<float> &b, int nv, int M, HsPacked &out)
+{
+    struct Node {
+        int id, t, R;
+    };
+    struct Warp {
+        int kind, q0, q1;
+    };
+    std::vector<Node> nodes[2];
+    std::vector<Warp> warps;  // HS_WARPS per CTA, empty ones with q0 = q1
+    out.desc.clear();
+    for (int kind = 1; kind >= 0; kind--) {  // the longer CTAs first
+        const int HM = hs_slots(kind);
+        std::vector<Node> &nd = nodes[kind];
+        nd.resize((size_t)nv);
+        for (int i = 0; i < nv; i++) {
+            int c = 0;
+            for (int k = 0; k < M; k++) c += b[(size_t)i * M + k] != 0.0f;
+            int t = 1;
+            while (t < 32 && (c + t - 1) / t + 2 > HM) t *= 2;
+            const int s = (c + t - 1) / t;
+            nd[i] = Node{i, t, std::min(HM, (s + 2 + 7) / 8 * 8)};
+        }
+        std::sort(nd.begin(), nd.end(), [](const Node &x, const Node &y) {
+            if (x.t != y.t) return x.t > y.t;
+            if (x.R != y.R) return x.R > y.R;
+            return x.id < y.id;
+        });
+        const size_t first = warps.size();
+        for (int q = 0; q < nv;) {
+            int e = q;
+            while (e < nv && nd[e].t == nd[q].t && e - q < 32 / nd[q].t) e++;
+            warps.push_back({kind, q, e});
+            q = e;
+        }
+        while ((warps.size() - first) % HS_WARPS) warps.push_back({kind, 0, 0});
+        for (size_t w = first; w < warps.size(); w += HS_WARPS) {
+            int R = 8;
+            for (int k = 0; k < HS_WARPS; k++)
+                if (warps[w + k].q1 > warps[w + k].q0) R = std::max(R, nd[warps[w + k].q0].R);
+            out.desc.push_back((uint8_t)(R / 8 | kind << 7));
+        }
+    }
+    const int nw = (int)warps.size();
+    out.chunks = nw / HS_WARPS;
+    out.tab.assign((size_t)nw * HS_ROWS * 32, 0u);
+    out.lane.assign((size_t)nw * 32, HS_NO_NODE);
+    const int nth = (int)std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+    std::atomic<int> next{0};
+    auto work = [&]() {
+        for (int w = next++; w < nw; w = next++) {
+            const Warp &wp = warps[w];
+            if (wp.q0 == wp.q1) continue;
+            std::vector<int> ids;
+            std::vector<std::vector<PackTrial>> tr;
+            for (int q = wp.q0; q < wp.q1; q++) {
+                const int i = nodes[wp.kind][q].id;
+                ids.push_back(i);
+                tr.emplace_back();
+                for (int k = 0; k < M; k++) {
+                    const size_t s = (size_t)i * M + k;
+                    if (b[s] == 0.0f) continue;
+                    const uint16_t g = (uint16_t)(idx[2 * s] & 0xffffu), l = (uint16_t)(idx[2 * s] >> 16),
+                                   m = (uint16_t)idx[2 * s + 1];
+                    tr.back().push_back(wp.kind ? PackTrial{{l, m}, b[s]} : PackTrial{{g, 0}, b[s]});
+                }
+            }
+            pack_warp(ids, tr, wp.kind, nodes[wp.kind][wp.q0].t, 8 * (out.desc[w / HS_WARPS] & 0x7f),
+                      0x9a175eedull + (uint64_t)w, &out.tab[(size_t)w * HS_ROWS * 32], &out.lane[(size_t)w * 32]);
+        }
+    };
+    std::vector<std::thread> pool;
+    for (int i = 1; i < nth; i++) pool.emplace_back(work);
+    work();
+    for (auto &th : pool) th.join();
+}
+
 void hs_free(HsTables &t, const DevFree &dfree)
 {
     if (t.d_idx) dfree(t.d_idx);
     if (t.d_b) dfree(t.d_b);
     if (t.d_xi) dfree(t.d_xi);
     if (t.d_jpk) dfree(t.d_jpk);
+    if (t.d_tab) dfree(t.d_tab);
+    if (t.d_lane) dfree(t.d_lane);
+    if (t.d_desc) dfree(t.d_desc);
     if (t.d_bc) dfree(t.d_bc);
+    if (t.d_pair) dfree(t.d_pair);
+    t.d_tab = t.d_lane = nullptr;
+    t.d_desc = nullptr;
+    t.d_pair = nullptr;
+    t.chunks = 0;
+    t.prep_cells = 0;
     t.d_idx = nullptr;
     t.d_b = nullptr;
     t.d_xi = nullptr;
@@ -439,21 +712,33 @@ int hs_build(HsTables &t, const int n[3], const double lo[3], const double h[3],
     }
     t.hh = 0.5 * h[0];
     for (int d = 0; d < 3; d++) t.half[d] = n[d] / 2;
-    t.d_idx = alloc(t.host_idx.size() * 4);
-    t.d_b = static_cast<float *>(alloc(t.host_b.size() * 4));
-    t.d_xi = static_cast<float *>(alloc(xf.size() * 4));
-    t.d_jpk = static_cast<uint32_t *>(alloc(jp.size() * 4));
-    if (!t.d_idx || !t.d_b || !t.d_xi || !t.d_jpk) { err = "device allocation (collision tables)"; return DVM_ENOMEM; }
-    std::vector<uint32_t> didx;
-    std::vector<float> db;
-    order_for_banks(t.host_idx, t.host_b, nv, trials, didx, db);
-    if (cudaMemcpy(t.d_idx, didx.data(), didx.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t.d_b, db.data(), db.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t.d_xi, xf.data(), xf.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t.d_jpk, jp.data(), jp.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+    // the device's copy of a table
+    auto put = [&](auto *&d, const auto &h) {
+        using T = typename std::remove_reference_t<decltype(h)>::value_type;
+        d = static_cast<std::remove_reference_t<decltype(d)>>(alloc(h.size() * sizeof(T)));
+        if (!d) return DVM_ENOMEM;
+        return cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess ? DVM_OK : DVM_ECUDA;
+    };
+    int rc = put(t.d_xi, xf);
+    if (!rc) rc = put(t.d_jpk, jp);
+    if (nv <= HS_PAIR_MAX_NV) {
+        HsPacked pk;
+        hs_pack(t.host_idx, t.host_b, nv, trials, pk);
+        if (!rc) rc = put(t.d_tab, pk.tab);
+        if (!rc) rc = put(t.d_lane, pk.lane);
+        if (!rc) rc = put(t.d_desc, pk.desc);
+        t.chunks = pk.chunks;
+    } else {
+        std::vector<uint32_t> didx;
+        std::vector<float> db;
+        order_for_banks(t.host_idx, t.host_b, nv, trials, didx, db);
+        if (!rc) rc = put(t.d_idx, didx);
+        if (!rc) rc = put(t.d_b, db);
+    }
+    if (rc) {
         cudaGetLastError();
-        err = "copy collision tables";
-        return DVM_ECUDA;
+        err = rc == DVM_ENOMEM ? "device allocation (collision tables)" : "copy collision tables";
+        return rc;
     }
     t.trials = trials;
     t.seed = seed;

@@ -21,13 +21,22 @@ struct HsTables {
     // weight b (= c).  A discarded trial keeps b = 0 and points at node i.
     std::vector<uint32_t> host_idx;   // [nv*trials][2]
     std::vector<float> host_b;        // [nv*trials]
-    void *d_idx = nullptr;
+    // gather tables: packed by warps for pairs of cells (chunks > 0), or in
+    // node order (idx, b)
+    int chunks = 0;                   // CTAs that hold the packed tables
+    uint32_t *d_tab = nullptr, *d_lane = nullptr;
+    uint8_t *d_desc = nullptr;
+    uint32_t *d_idx = nullptr;
     float *d_b = nullptr;
     float *d_xi = nullptr;            // node velocities [3][nv], FP32
     uint32_t *d_jpk = nullptr;        // per node: xi_d = hh j_d, j_d odd, packed as bytes j_d + 64
     double hh = 0.0;                  // half the velocity spacing (the same on every axis)
     int half[3] = {0, 0, 0};          // nodes per axis / 2 (the grid's sign-group shape)
-    float *d_bc = nullptr;            // scratch: B and C of every cell [ncells][nv][2]
+    // scratch for bc_cells cells at a time: B and C, [2][bc_cells][nv], and f
+    // as pairs of cells, [bc_cells / 2][nv][2] (packed tables)
+    float *d_bc = nullptr;
+    float *d_pair = nullptr;
+    int64_t prep_cells = 0;           // the mesh size the scratch was made for
     int64_t bc_cells = 0;
 };
 
@@ -48,7 +57,33 @@ int hs_build(HsTables &t, const int n[3], const double lo[3], const double h[3],
 int64_t korobov_multiplier(int64_t M);
 void hs_free(HsTables &t, const DevFree &dfree);
 
-// Per-cell scratch for ncells cells (B, C and the correction sums).
+// The weighted trials packed for the gather kernel on pairs of cells.  Two
+// kinds of warp: kind 0 holds the partners gamma for the sums B (Eq. 4), kind
+// 1 the post-collision nodes l, m for the sums C (Eq. 5).  A warp's 96 rows of
+// 32 words (one word per lane):
+//   kind 0: 32 rows of two partners (slots 2r, 2r + 1), then 64 rows of b;
+//   kind 1: 48 rows of (l, m), then 48 rows of b;
+// two nodes x, y in a word as x << 3 | y << 17 (x << 3 is the byte offset in a
+// tile of 8-byte pairs).
+constexpr int HS_WARPS = 16;          // warps per CTA of the gather kernel
+constexpr int HS_ROWS = 96;
+constexpr uint32_t HS_NO_NODE = 0xfffffu;
+constexpr int hs_slots(int kind) { return kind == 0 ? 64 : 48; }
+struct HsPacked {
+    int chunks = 0;                // CTAs
+    std::vector<uint32_t> tab;     // [chunks * HS_WARPS][HS_ROWS][32]
+    std::vector<uint32_t> lane;    // [chunks * HS_WARPS][32]: node (HS_NO_NODE: none) | log2(lanes of the node) << 20
+    std::vector<uint8_t> desc;     // [chunks]: groups of eight slots that its warps run | kind << 7
+};
+void hs_pack(const std::vector<uint32_t> &idx, const std::vector<float> &b, int nv, int M, HsPacked &out);
+
+// Largest grid of the pair kernel: two stages of 8 nv bytes beside its own
+// few bytes of shared memory, and node offsets of 17 bits.  Larger grids (up
+// to 25,600 nodes) run one cell at a time: a pair's tile would fill shared
+// memory alone, and its copy could not overlap the gathers.
+constexpr int HS_PAIR_MAX_NV = 14336;
+
+// Scratch for batches of cells (B, C and the cells' f as pairs), at most 4 GB.
 int hs_prepare(HsTables &t, int64_t ncells, const DevAlloc &alloc, const DevFree &dfree);
 
 // f (storage precision, already holding f* from the transport launch) is

@@ -6,13 +6,16 @@
 // gathers f across cells from a velocity-major copy; here the roles are
 // swapped to keep every gather on chip:
 //
-//  k_hs_bc   table-stationary: a CTA holds the trials of 64 nodes (256
-//            threads) or, on grids of more than 6144 nodes, 128 nodes (512
-//            threads) in registers (32 per thread) and streams cells through a
-//            double-buffered shared-memory tile, each tile a single bulk
-//            copy (cp.async.bulk, completion on an mbarrier).  It writes
-//            B_i = sum_k b f_gamma (Eq. 4) and C_i = sum_k c f_l f_m (Eq. 5)
-//            for its nodes to a per-cell scratch array.
+//  k_hs_pairs   interleaves the f of two cells, so that one 64-bit gather
+//            serves both;
+//  k_hs_gather  table-stationary: a CTA of 512 threads holds the weighted
+//            trials of some nodes in registers (64 or 48 per thread) and
+//            streams pairs of cells through two shared-memory tiles, each a
+//            single bulk copy (cp.async.bulk, completion on an mbarrier).  It
+//            writes B_i = sum_k b f_gamma (Eq. 4) or C_i = sum_k c f_l f_m
+//            (Eq. 5) for its nodes to per-cell scratch arrays.
+//  k_hs_bc   the same sums one cell at a time, for grids whose pair tiles do
+//            not fit in shared memory twice (more than 14,336 nodes).
 //  k_hs_corr per cell: the five coefficients of P (Eq. 6) from the moment
 //            system, its sums formed exactly in an integer basis and
 //            carried in double-float, solved in FP64 in the centred basis
@@ -36,15 +39,190 @@ void count_launch();
 
 namespace {
 
-constexpr int HE = 32;    // trials held per thread
+constexpr int HE = 32;    // trials held per thread of k_hs_bc
+constexpr int HT = 512;   // threads per CTA of k_hs_bc
 constexpr int CT = 256;   // threads per CTA of k_hs_corr
 
-// HT threads per CTA (256 or 512; at most 128 registers a thread either way)
-template <int HT>
-__global__ void __launch_bounds__(HT, 512 / HT)
-    k_hs_bc(const float *__restrict__ fs, float2 *__restrict__ bc, int64_t ncells, int nv, int M,
-            const uint2 *__restrict__ idx, const float *__restrict__ bw, int64_t cells_per_cta,
-            const int32_t *__restrict__ list, const int *__restrict__ count, int *status)
+// The rows of a batch: rows r0, r0 + 1, .. (at most nb) of the cells, or of
+// a device list of cells.
+struct Rows {
+    int64_t r0, nb, ncells;
+    const int32_t *list;  // may be null
+    const int *n;         // entries of the list
+    __device__ int64_t count() const
+    {
+        const int64_t left = (list ? (int64_t)*n : ncells) - r0;
+        return left < 0 ? 0 : left < nb ? left : nb;
+    }
+    __device__ int64_t cell(int64_t r) const { return list ? (int64_t)list[r0 + r] : r0 + r; }
+};
+
+// f of the batch's rows as pairs: out [row / 2][nv][2]; the missing partner
+// of an odd last row is zero.  HBM-bound: 12,016 cells x 24^3 (1.33 GB read
+// and written) in 199 us, 3% of the gather kernel's time.
+__global__ void __launch_bounds__(256) k_hs_pairs(const float *__restrict__ f, float4 *__restrict__ out, Rows rw, int nv)
+{
+    const int64_t n = rw.count(), r = 2 * (int64_t)blockIdx.x;
+    if (r >= n) return;
+    const bool two = r + 1 < n;
+    const float4 *a = reinterpret_cast<const float4 *>(f + rw.cell(r) * nv);
+    const float4 *b = reinterpret_cast<const float4 *>(f + rw.cell(two ? r + 1 : r) * nv);
+    float4 *o = out + (int64_t)blockIdx.x * (nv / 2);
+    for (int q = threadIdx.x; q < nv / 4; q += blockDim.x) {
+        const float4 x = __ldg(a + q);
+        float4 y = __ldg(b + q);
+        if (!two) y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        o[2 * q] = make_float4(x.x, y.x, x.y, y.y);
+        o[2 * q + 1] = make_float4(x.z, y.z, x.w, y.w);
+    }
+}
+
+// ---------------------------------------------------------------- pairs of cells
+// What bounds it: the shared-memory pipe.  A trial costs one (B) or two (C)
+// 64-bit gathers for two cells; a warp's gather takes two wavefronts without
+// conflicts and about 2.6 with the order that hs_pack finds, against 1.5
+// instruction issue cycles, and each pair's tile costs its own write into
+// shared memory.  The 96 registers a thread holds of the table set how many
+// nodes a tile serves.
+constexpr int GT = 32 * HS_WARPS;                 // threads of k_hs_gather
+constexpr uint32_t STAGE = 8u * HS_PAIR_MAX_NV;  // distance of the two tiles
+
+struct GatherArgs {
+    const float2 *pairs;
+    float *out[2];  // B and C planes, [rows][nv]
+    Rows rw;
+    int nv, chunks;
+    const uint32_t *tab, *lane;
+    const uint8_t *desc;
+    int *status;
+};
+
+__device__ inline float2 lds_pair(uint32_t addr)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+
+// The pairs p0 .. p1 - 1 on one warp of kind KIND with 8 NG slots.  The last
+// warp to leave a tile refills it with the pair after next, so no warp waits
+// for another but through the tiles.
+template <int KIND, int NG>
+__device__ __forceinline__ void gather_pairs(const GatherArgs &g, int warp, int p0, int np, bool odd, uint32_t tile,
+                                             uint64_t *full, int *left)
+{
+    constexpr int SL = 8 * NG, BROW = HS_ROWS - hs_slots(KIND);
+    constexpr uint32_t MASK = 0x1fff8u;
+    const int lane = threadIdx.x & 31;
+    const uint32_t *tb = g.tab + (int64_t)warp * (HS_ROWS * 32) + lane;
+    uint32_t w[KIND ? SL : SL / 2];
+    float b[SL];
+#pragma unroll
+    for (int e = 0; e < (KIND ? SL : SL / 2); e++) w[e] = __ldg(tb + 32 * e);
+#pragma unroll
+    for (int e = 0; e < SL; e++) b[e] = __uint_as_float(__ldg(tb + 32 * (BROW + e)));
+    const uint32_t lt = __ldg(g.lane + (int64_t)warp * 32 + lane);
+    const uint32_t node = lt & 0xfffffu;
+    const int t = 1 << (lt >> 20);
+    const bool writes = node != HS_NO_NODE && (lane & (t - 1)) == 0;
+    float *out = g.out[KIND] + 2 * (int64_t)p0 * g.nv + node;
+    for (int p = 0; p < np; p++) {
+        const int s = p & 1;
+        const uint32_t base = tile + (s ? STAGE : 0u);
+        if (!mbar_wait(&full[s], (uint32_t)(p >> 1) & 1u)) {
+            // a tile never arrived: report, and leave no copy in flight behind
+            // (the other tile's is the next pair's, if there is one)
+            if (lane == 0) atomicOr(g.status, ST_TIMEOUT);
+            mbar_wait(&full[s], (uint32_t)(p >> 1) & 1u);
+            if (p + 1 < np) mbar_wait(&full[s ^ 1], (uint32_t)((p + 1) >> 1) & 1u);
+            return;
+        }
+        float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int e = 0; e < SL; e++) {
+            // keep the offsets' extraction inside the loop (hoisted, the
+            // extracted offsets would need another 32 to 48 registers)
+            if (KIND == 1 || (e & 1) == 0) asm volatile("" : "+r"(w[KIND ? e : e / 2]));
+            if constexpr (KIND == 0) {
+                const uint32_t at = (e & 1) ? (w[e / 2] >> 14) & MASK : w[e / 2] & MASK;
+                const float2 v = lds_pair(base + at);
+                acc.x = fmaf(b[e], v.x, acc.x);
+                acc.y = fmaf(b[e], v.y, acc.y);
+            } else {
+                const float2 l = lds_pair(base + (w[e] & MASK)), m = lds_pair(base + ((w[e] >> 14) & MASK));
+                const float2 v = __fmul2_rn(l, m);
+                acc.x = fmaf(b[e], v.x, acc.x);
+                acc.y = fmaf(b[e], v.y, acc.y);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence_block();
+            if (atomicAdd(&left[s], 1) == HS_WARPS - 1) {
+                __threadfence_block();
+                left[s] = 0;
+                if (p + 2 < np) {
+                    mbar_expect_tx(&full[s], 8u * (uint32_t)g.nv);
+                    bulk_g2s_addr(base, g.pairs + (int64_t)(p0 + p + 2) * g.nv, 8u * (uint32_t)g.nv, &full[s]);
+                }
+            }
+        }
+        for (int m = 1; m < t; m <<= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, m);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, m);
+        }
+        if (writes) {
+            out[0] = acc.x;
+            if (p + 1 < np || !odd) out[g.nv] = acc.y;
+        }
+        out += 2 * (int64_t)g.nv;
+    }
+}
+
+// CTA (segment, chunk): the nodes of a chunk of the tables for a segment of
+// the batch's pairs.
+__global__ void __launch_bounds__(GT, 1) k_hs_gather(const GatherArgs g)
+{
+    extern __shared__ __align__(128) unsigned char gtile[];  // two tiles, STAGE apart
+    __shared__ __align__(8) uint64_t full[2];
+    __shared__ int left[2];
+    const int nrows = (int)g.rw.count(), npairs = (nrows + 1) / 2;  // a batch is below 2^31 rows
+    const int nseg = gridDim.x / g.chunks, per = (npairs + nseg - 1) / nseg;
+    const int p0 = (int)(blockIdx.x / g.chunks) * per, np = min(per, npairs - p0);
+    if (np <= 0) return;
+    const bool odd = (nrows & 1) && p0 + np == npairs;  // the last pair has one cell
+    const int chunk = blockIdx.x % g.chunks;
+    const uint32_t tile = smem_u32(gtile);
+    if (threadIdx.x == 0) {
+        mbar_init(&full[0], 1);
+        mbar_init(&full[1], 1);
+        left[0] = left[1] = 0;
+        mbar_fence_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t bytes = 8u * (uint32_t)g.nv;
+        for (int s = 0; s < 2 && s < np; s++) {
+            mbar_expect_tx(&full[s], bytes);
+            bulk_g2s_addr(tile + (s ? STAGE : 0u), g.pairs + (int64_t)(p0 + s) * g.nv, bytes, &full[s]);
+        }
+    }
+    const int warp = chunk * HS_WARPS + (threadIdx.x >> 5);
+#define DVM_RUN(K, N) \
+    case (K << 7 | N): gather_pairs<K, N>(g, warp, p0, np, odd, tile, full, left); break;
+    switch (g.desc[chunk]) {
+        DVM_RUN(0, 1) DVM_RUN(0, 2) DVM_RUN(0, 3) DVM_RUN(0, 4)
+        DVM_RUN(0, 5) DVM_RUN(0, 6) DVM_RUN(0, 7) DVM_RUN(0, 8)
+        DVM_RUN(1, 1) DVM_RUN(1, 2) DVM_RUN(1, 3) DVM_RUN(1, 4) DVM_RUN(1, 5) DVM_RUN(1, 6)
+    }
+#undef DVM_RUN
+    // the copies issued ahead have all been waited for (or given up on) above
+}
+
+// ---------------------------------------------------------------- one cell at a time
+__global__ void __launch_bounds__(HT, 1)
+    k_hs_bc(const float *__restrict__ fs, float *__restrict__ Bp, float *__restrict__ Cp, Rows rw, int nv, int M,
+            const uint2 *__restrict__ idx, const float *__restrict__ bw, int *status)
 {
     extern __shared__ __align__(128) float tile[];  // [2][nv]
     __shared__ __align__(8) uint64_t bar[2];
@@ -65,15 +243,12 @@ __global__ void __launch_bounds__(HT, 512 / HT)
         w1[e] = t.y;
         b[e] = valid ? bw[e0 + e] : 0.0f;
     }
-    // rows c0..c1-1 of this CTA: cells, or entries of the cell list
-    int64_t nrows = ncells, per = cells_per_cta;
-    if (list) {
-        nrows = *count;
-        per = (nrows + gridDim.y - 1) / gridDim.y;
-    }
+    // rows c0..c1-1 of the batch for this CTA
+    const int64_t nrows = rw.count();
+    const int64_t per = (nrows + gridDim.y - 1) / gridDim.y;
     const int64_t c0 = (int64_t)blockIdx.y * per;
     const int64_t c1 = c0 + per < nrows ? c0 + per : nrows;
-    auto src = [&](int64_t r) { return fs + (list ? (int64_t)list[r] : r) * nv; };
+    auto src = [&](int64_t r) { return fs + rw.cell(r) * nv; };
     const uint32_t bytes = (uint32_t)nv * 4u;
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -118,7 +293,10 @@ __global__ void __launch_bounds__(HT, 512 / HT)
             B += __shfl_xor_sync(0xffffffffu, B, m);
             C += __shfl_xor_sync(0xffffffffu, C, m);
         }
-        if (valid && tid % tpn == 0) bc[c * nv + node] = make_float2(B, C);
+        if (valid && tid % tpn == 0) {
+            Bp[c * nv + node] = B;
+            Cp[c * nv + node] = C;
+        }
         __syncthreads();
         if (abort_flag) {
             // a tile never arrived: report, give the copies in flight a bounded
@@ -169,18 +347,18 @@ constexpr int NSUM = 20;  // 15 distinct entries of the moment matrix, 5 gain mo
 // serial solve (C4: 7.56 -> 7.29 ms per step; two or four CTAs were slower on
 // one of the 16^3 and 24^3 grids)
 __global__ void __launch_bounds__(CT, 3)
-    k_hs_corr(float *__restrict__ f, const float2 *__restrict__ bc, const float *__restrict__ xi3,
+    k_hs_corr(float *__restrict__ f, const float *__restrict__ Bp, const float *__restrict__ Cp,
+              const float *__restrict__ xi3,
               const uint32_t *__restrict__ jpk, double hh, double dV, const double *__restrict__ mom, int nv,
-              int3 half, float dtkn, const int32_t *__restrict__ list, const int *__restrict__ count,
-              float *__restrict__ q_out, double *__restrict__ res, int *status)
+              int3 half, float dtkn, Rows rw, float *__restrict__ q_out, double *__restrict__ res, int *status)
 {
     __shared__ ffn part[NSUM][CT];
     __shared__ double S[NSUM];
     __shared__ float sd[5];
     // row blockIdx.x of B and C belongs to this cell (an entry of the list, if any)
     const int64_t row = blockIdx.x;
-    if (list && row >= (int64_t)*count) return;
-    const int64_t cell = list ? (int64_t)list[row] : row;
+    if (row >= rw.count()) return;
+    const int64_t cell = rw.cell(row);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const double *mo = mom + cell * 5;
     const double rho = mo[0], Td = mo[4];
@@ -194,7 +372,7 @@ __global__ void __launch_bounds__(CT, 3)
         return;
     }
     float *fc = f + cell * (int64_t)nv;
-    const float2 *bcc = bc + row * (int64_t)nv;
+    const float *Bc = Bp + row * (int64_t)nv, *Cc = Cp + row * (int64_t)nv;
     // The sums over the nodes, pencil by pencil: a pencil is the line of nodes
     // along z at fixed (x, y) node indices, both z signs (sign groups 2 o_xy
     // and 2 o_xy + 1, positions pos .. pos + hz - 1 in each).  Along a pencil
@@ -225,7 +403,7 @@ __global__ void __launch_bounds__(CT, 3)
             for (int m = 0; m < half.z; m++) {
                 const int v = v0 + m;
                 const float fv = fc[v];
-                const float2 q = bcc[v];
+                const float2 q = make_float2(Bc[v], Cc[v]);
                 const float jz = (float)((int)((jpk[v] >> 16) & 0xffu) - 64);
                 const float jz2 = jz * jz;
                 const float w = fv * q.x, wl = fmaf(fv, q.x, -w);  // f B = w + wl exactly
@@ -369,7 +547,7 @@ __global__ void __launch_bounds__(CT, 3)
     float worst = 0.0f;
     for (int v = tid; v < nv; v += CT) {
         const float fv = fc[v];
-        const float2 q = bcc[v];
+        const float2 q = make_float2(Bc[v], Cc[v]);
         const float cx = (xi3[v] - ux) * ist, cy = (xi3[nv + v] - uy) * ist, cz = (xi3[2 * nv + v] - uz) * ist;
         const float P = 1.0f + d0 + dx * cx + dy * cy + dz * cz + d4 * (cx * cx + cy * cy + cz * cz - 3.0f);
         const float loss = P * q.x;
@@ -389,14 +567,30 @@ bool hs_trials_supported(int trials)
     return tpn <= 32 && (tpn & (tpn - 1)) == 0;
 }
 
+// Rows of one batch: scratch of 8 nv bytes a row for B and C and, for the
+// pair kernel, 4 nv for f as pairs, 4 GB at most (24k cells at 24^3, enough to
+// fill the GPU many times over; the scratch of a whole mesh would be three
+// times its f).
+static int64_t batch_rows(int64_t ncells, int nv, size_t bytes)
+{
+    const int64_t cap = std::max<int64_t>(2, (int64_t)(bytes / ((size_t)nv * 12)) & ~(int64_t)1);
+    return std::min(cap, (ncells + 1) & ~(int64_t)1);
+}
+
 int hs_prepare(HsTables &t, int64_t ncells, const DevAlloc &alloc, const DevFree &dfree)
 {
     if (!t.ready) return DVM_ESTATE;
-    if (t.d_bc && t.bc_cells == ncells) return DVM_OK;
+    if (t.d_bc && t.prep_cells == ncells) return DVM_OK;
     if (t.d_bc) dfree(t.d_bc);
-    t.d_bc = static_cast<float *>(alloc((size_t)ncells * t.nv * 2 * sizeof(float)));
-    t.bc_cells = t.d_bc ? ncells : 0;
-    return t.d_bc ? DVM_OK : DVM_ENOMEM;
+    if (t.d_pair) dfree(t.d_pair);
+    t.d_bc = t.d_pair = nullptr;
+    t.prep_cells = 0;
+    t.bc_cells = batch_rows(ncells, t.nv, (size_t)4 << 30);
+    t.d_bc = static_cast<float *>(alloc((size_t)t.bc_cells * t.nv * 2 * sizeof(float)));
+    if (t.chunks) t.d_pair = static_cast<float *>(alloc((size_t)t.bc_cells * t.nv * sizeof(float)));
+    if (!t.d_bc || (t.chunks && !t.d_pair)) return DVM_ENOMEM;
+    t.prep_cells = ncells;
+    return DVM_OK;
 }
 
 // Cell splits of the k_hs_bc grid (node chunks x cell ranges): at least two
@@ -421,74 +615,88 @@ static int64_t hs_splits(int chunks, int slots, int64_t ncells)
     return std::max<int64_t>(1, std::min<int64_t>(best, ncells));
 }
 
-// The launch shape of k_hs_bc for nv nodes and ncells rows.  Each CTA streams
-// the whole f of every cell of its range through shared memory for the trials
-// of its nodes, so the tile is worth 3 M npc / nv gathers per loaded value:
-// 1.8 at 24^3 with 64 nodes per CTA, 3.6 with 128.  Grids of more than 6144
-// nodes take 512 threads (128 nodes), the others 256 (measured: 24^3, 543.9 ->
-// 389.8 ms per step on the 253k-cell flow; 16^3 is 1.5% faster with 256).
-// Every check that can refuse the launch is made here, before anything is
-// queued.
+// The launch of the B and C sums for batches of nb rows (the last may be
+// shorter).  Every check that can refuse it is made here, before anything is
+// queued.  Pair kernel: each CTA takes one chunk of the tables and a segment
+// of the pairs; loading its tables costs about as much as three pairs, and
+// CTAs are handed out as SMs come free, so that with W pair steps an SM a
+// segment of sqrt(6 W) pairs balances the two (3 W / L against half a segment
+// at the end).
 struct BcLaunch {
-    int threads = 0;
     dim3 grid;
     size_t dyn = 0;
-    int64_t per = 0;  // rows per CTA
+    int64_t nb = 0;
 };
 
-static int bc_plan(const HsTables &t, int nv, int64_t ncells, BcLaunch &L)
+static int bc_plan(const HsTables &t, int nv, int64_t nb, BcLaunch &L)
 {
-    const int ht = nv > 6144 ? 512 : 256;
-    const int tpn = t.trials / HE, npc = ht / tpn;
-    const int chunks = (nv + npc - 1) / npc;
-    const size_t dyn = 2 * (size_t)nv * sizeof(float);
-    if (dyn > 200 * 1024) return DVM_ENOTIMPL;
-    auto kern = ht == 512 ? k_hs_bc<512> : k_hs_bc<256>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
-        return DVM_ECUDA;
     int dev = 0, nsm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, ht, dyn) != cudaSuccess || occ < 1)
+    L.nb = nb;
+    if (t.chunks) {
+        L.dyn = STAGE + 8 * (size_t)nv;
+        if (cudaFuncSetAttribute(k_hs_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * STAGE)) !=
+            cudaSuccess)
+            return DVM_ECUDA;
+        const int64_t pairs = (nb + 1) / 2;
+        const double W = (double)pairs * t.chunks / nsm;
+        int64_t len = std::max<int64_t>(1, (int64_t)std::sqrt(6.0 * W));
+        len = std::min(len, std::max<int64_t>(1, pairs * t.chunks / nsm));
+        L.grid = dim3((unsigned)(t.chunks * ((pairs + len - 1) / len)));
+        return DVM_OK;
+    }
+    const int tpn = t.trials / HE, npc = HT / tpn;
+    const int chunks = (nv + npc - 1) / npc;
+    L.dyn = 2 * (size_t)nv * sizeof(float);
+    if (L.dyn > 200 * 1024) return DVM_ENOTIMPL;
+    if (cudaFuncSetAttribute(k_hs_bc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+        return DVM_ECUDA;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hs_bc, HT, L.dyn) != cudaSuccess || occ < 1)
         return DVM_ENOTIMPL;
-    int64_t splits = hs_splits(chunks, nsm * occ, ncells);
-    L.per = (ncells + splits - 1) / splits;
-    splits = (ncells + L.per - 1) / L.per;
-    L.threads = ht;
-    L.grid = dim3((unsigned)chunks, (unsigned)splits);
-    L.dyn = dyn;
+    L.grid = dim3((unsigned)chunks, (unsigned)hs_splits(chunks, nsm * occ, nb));
     return DVM_OK;
 }
 
-static int bc_launch(const BcLaunch &L, const HsTables &t, const float *f, float2 *bc, int64_t ncells, int nv,
-                     const int32_t *list, const int *count, cudaStream_t s, int *status)
+// What an update needs beside its rows.
+struct CorrArgs {
+    double dV;
+    const double *mom;
+    float dtkn;
+    float *q_out;
+    double *res;
+};
+
+// B, C and the correction, batch by batch.
+static int run_batches(const BcLaunch &L, const HsTables &t, float *f, float *bc, float *pair, int nv, int64_t ncells,
+                       const int32_t *list, const int *count, const CorrArgs &c, cudaStream_t s, int *status)
 {
-    const uint2 *idx = static_cast<const uint2 *>(t.d_idx);
-    if (L.threads == 512)
-        k_hs_bc<512><<<L.grid, 512, L.dyn, s>>>(f, bc, ncells, nv, t.trials, idx, t.d_b, L.per, list, count, status);
-    else
-        k_hs_bc<256><<<L.grid, 256, L.dyn, s>>>(f, bc, ncells, nv, t.trials, idx, t.d_b, L.per, list, count, status);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
+    float *Bp = bc, *Cp = bc + L.nb * nv;
+    for (int64_t r0 = 0; r0 < ncells; r0 += L.nb) {
+        const Rows rw{r0, L.nb, ncells, list, count};
+        const unsigned rows = (unsigned)std::min(L.nb, ncells - r0);
+        if (t.chunks) {
+            k_hs_pairs<<<(rows + 1) / 2, 256, 0, s>>>(f, reinterpret_cast<float4 *>(pair), rw, nv);
+            count_launch();
+            const GatherArgs g{reinterpret_cast<const float2 *>(pair), {Bp, Cp}, rw, nv, t.chunks, t.d_tab, t.d_lane,
+                               t.d_desc, status};
+            k_hs_gather<<<L.grid, GT, L.dyn, s>>>(g);
+        } else {
+            k_hs_bc<<<L.grid, HT, L.dyn, s>>>(f, Bp, Cp, rw, nv, t.trials, reinterpret_cast<const uint2 *>(t.d_idx),
+                                              t.d_b, status);
+        }
+        count_launch();
+        k_hs_corr<<<rows, CT, 0, s>>>(f, Bp, Cp, t.d_xi, t.d_jpk, t.hh, c.dV, c.mom, nv,
+                                      make_int3(t.half[0], t.half[1], t.half[2]), c.dtkn, rw, c.q_out, c.res, status);
+        count_launch();
+        if (cudaGetLastError() != cudaSuccess) return DVM_ECUDA;
+    }
+    return DVM_OK;
 }
 
 int launch_hs_collide(HsTables &t, const StepParams &p, void *f, double kn, double dt)
 {
-    if (p.prec != DVM_F32) return DVM_ENOTIMPL;
-    if (!t.ready || t.nv != p.nv || !t.d_bc) return DVM_ESTATE;
-    BcLaunch L;
-    int rc = bc_plan(t, p.nv, p.ncells, L);
-    if (!rc)
-        rc = bc_launch(L, t, static_cast<const float *>(f), reinterpret_cast<float2 *>(t.d_bc), p.ncells, p.nv,
-                       nullptr, nullptr, p.stream, p.status);
-    if (rc) return rc;
-    k_hs_corr<<<(unsigned)p.ncells, CT, 0, p.stream>>>(static_cast<float *>(f),
-                                                      reinterpret_cast<const float2 *>(t.d_bc), t.d_xi, t.d_jpk,
-                                                      t.hh, p.dV, p.mom_out, p.nv,
-                                                      make_int3(t.half[0], t.half[1], t.half[2]), (float)(dt / kn),
-                                                      nullptr, nullptr, nullptr, p.res_out, p.status);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
+    return launch_hs_general(t, p, static_cast<float *>(f), nullptr, nullptr, nullptr, kn, dt);
 }
 
 // The update on the cells of a device list only (*count entries, at most
@@ -497,21 +705,13 @@ int launch_hs_general(HsTables &t, const StepParams &p, float *f, const int32_t 
                       float *q_out, double kn, double dt)
 {
     if (p.prec != DVM_F32) return DVM_ENOTIMPL;
-    if (!t.ready || t.nv != p.nv || !t.d_bc || t.bc_cells < p.ncells) return DVM_ESTATE;
+    if (!t.ready || t.nv != p.nv || !t.d_bc || t.prep_cells < p.ncells) return DVM_ESTATE;
     if (p.ncells <= 0) return DVM_OK;
     BcLaunch L;
-    int rc = bc_plan(t, p.nv, p.ncells, L);
-    if (!rc)
-        rc = bc_launch(L, t, f, reinterpret_cast<float2 *>(t.d_bc), p.ncells, p.nv, list, count, p.stream,
-                       p.status);
+    const int rc = bc_plan(t, p.nv, t.bc_cells, L);
     if (rc) return rc;
-    k_hs_corr<<<(unsigned)p.ncells, CT, 0, p.stream>>>(f, reinterpret_cast<const float2 *>(t.d_bc), t.d_xi,
-                                                      t.d_jpk, t.hh, p.dV, p.mom_out, p.nv,
-                                                      make_int3(t.half[0], t.half[1], t.half[2]),
-                                                      q_out ? 0.0f : (float)(dt / kn), list, count, q_out,
-                                                      q_out ? nullptr : p.res_out, p.status);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
+    const CorrArgs c{p.dV, p.mom_out, q_out ? 0.0f : (float)(dt / kn), q_out, q_out ? nullptr : p.res_out};
+    return run_batches(L, t, f, t.d_bc, t.d_pair, p.nv, p.ncells, list, count, c, p.stream, p.status);
 }
 
 // ---------------------------------------------------------------- allocation-free variant
@@ -587,26 +787,23 @@ int launch_hs_collide_noalloc(HsTables &t, const StepParams &p, float *f, const 
 {
     if (p.prec != DVM_F32) return DVM_ENOTIMPL;
     if (!t.ready || t.nv != p.nv) return DVM_ESTATE;
-    const size_t need_bc = (size_t)p.ncells * p.nv * 2 * sizeof(float);
-    if (need_bc + (size_t)p.ncells * 5 * sizeof(double) > NOALLOC_BYTES) return DVM_EINVAL;
-    // every check comes before the first launch, so that a refusal queues no work
+    const size_t mom_bytes = (size_t)p.ncells * 5 * sizeof(double);
+    if ((size_t)p.ncells * p.nv * 2 * sizeof(float) + mom_bytes > NOALLOC_BYTES) return DVM_EINVAL;
+    // every check comes before the first launch, so that a refusal queues no
+    // work.  At the scratch limit the pairs of f leave room for two thirds of
+    // the rows: two batches.
     BcLaunch L;
-    int rc = bc_plan(t, p.nv, p.ncells, L);
+    int rc = bc_plan(t, p.nv, batch_rows(p.ncells, p.nv, NOALLOC_BYTES - mom_bytes - 64), L);
     if (rc) return rc;
     void *base = nullptr;
     rc = noalloc_scratch(&base);
     if (rc) return rc;
-    float *bc = static_cast<float *>(base);
-    double *mom = reinterpret_cast<double *>(static_cast<unsigned char *>(base) + need_bc);
+    float *bc = static_cast<float *>(base), *pair = bc + (size_t)L.nb * p.nv * 2;
+    double *mom = reinterpret_cast<double *>(static_cast<unsigned char *>(base) + (NOALLOC_BYTES - mom_bytes) / 64 * 64);
     rc = launch_moments(DVM_F32, f, p.ncells, g, mom, p.stream);
     if (rc) return rc;
-    rc = bc_launch(L, t, f, reinterpret_cast<float2 *>(bc), p.ncells, p.nv, nullptr, nullptr, p.stream, p.status);
-    if (rc) return rc;
-    k_hs_corr<<<(unsigned)p.ncells, CT, 0, p.stream>>>(f, reinterpret_cast<const float2 *>(bc), t.d_xi, t.d_jpk,
-                                                      t.hh, g.dV, mom, p.nv, make_int3(t.half[0], t.half[1], t.half[2]),
-                                                      (float)(dt / kn), nullptr, nullptr, nullptr, nullptr, p.status);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
+    const CorrArgs c{g.dV, mom, (float)(dt / kn), nullptr, nullptr};
+    return run_batches(L, t, f, bc, pair, p.nv, p.ncells, nullptr, nullptr, c, p.stream, p.status);
 }
 
 }  // namespace dvm
