@@ -119,6 +119,11 @@ __device__ inline void cp_async8(void *dst, const void *src, uint32_t dep)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8; // %2" ::"r"(smem_u32(dst)), "l"(src), "r"(dep)
                  : "memory");
 }
+// 16 bytes, of which the first `bytes` (0 or 16) are read and the rest is zero
+__device__ inline void cp_async16_zfill(uint32_t dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
 // Prefetch of the line holding src into L2.
 __device__ inline void prefetch_l2(const void *src) { asm volatile("prefetch.global.L2 [%0];" ::"l"(src)); }
 

@@ -2,15 +2,24 @@
 // SiLU hidden activations, BF16 weights and activations, FP32 accumulation,
 // run and trained on the 5th-generation tensor cores.
 //
-// Every contraction is one kernel, C[M x N] = A[M x K] . B[N x K]^T with both
-// operands BF16 and K contiguous in global memory: a CTA owns 128 rows of C,
-// stages 64-wide K chunks of A and B into shared memory in the 128-byte
-// swizzled K-major layout (two stages), one thread issues tcgen05.mma
-// (M = 128, N <= 256, K = 16 per instruction) into a tensor-memory
-// accumulator, and the four warps read their 32 rows back with tcgen05.ld
-// for a fused epilogue (bias, SiLU, BF16 rounding, transposed copies).
-// Forward, backward (weight gradients as C = dZ^T-by-activation products)
-// and the Adam update all run on the device.
+// Every contraction is C[M x N] = A[M x K] . B[N x K]^T with both operands BF16
+// and K contiguous in global memory: a CTA owns 128 rows of C, stages 64-wide K
+// chunks of A and B into a four-deep shared-memory ring with cp.async in the
+// 128-byte swizzled K-major layout, one thread issues tcgen05.mma (M = 128,
+// N <= 256, K = 16 per instruction) into a tensor-memory accumulator, and the
+// eight warps read it back with tcgen05.ld for a fused epilogue: bias, SiLU and
+// the transposed copies of the forward pass; the output gradient with loss and
+// bias-gradient sums; the SiLU derivative of the backward pass.  The weight
+// gradients (C = dZ^T . activation, long K) of all four layers are one launch,
+// split over K.  Forward, backward and the Adam update all run on the device.
+//
+// Bound by the latency of a few dependent chunks per launch (the network is
+// 3.1 GFLOP a pass at 24k rows): with 16-byte loads through registers, two
+// stages and 128 threads a 256 x 256 layer took 52 us on 24,032 rows, 38 us on
+// 8,192, and the weight gradients, on two CTAs each, most of a gradient's
+// 2.9 ms.  Now 14 us (24,032 rows, inference), 20 to 23 us with the transposed copies of
+// training (8,192 rows), and 15 us for all weight gradients; the whole gradient
+// takes 9 launches instead of 24.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -20,6 +29,7 @@
 
 #include "../../include/dvm.h"
 #include "async.cuh"
+#include "common.cuh"
 #include "kernels.hpp"
 #include "mlp.hpp"
 #include "tc.cuh"
@@ -30,8 +40,18 @@ void count_launch();
 
 namespace {
 
-constexpr int GT = 128;             // threads per GEMM CTA
+constexpr int GT = 256;             // threads per GEMM CTA
+constexpr int NSTAGE = 4;
 constexpr uint32_t STAGE_A = 16384; // 128 rows x 128 bytes
+constexpr uint32_t STAGE_BYTES = STAGE_A + 32768;
+
+// what the epilogue makes of the accumulator v
+enum {
+    EP_FORWARD,  // z = v + bias: Cf = z, H = act(z) and its transposed copy
+    EP_OUT,      // r = v + bias - T: H = d = scale r and its transposed copy, sums of d and of r^2
+    EP_BACK,     // H = d = v silu'(Z) and its transposed copy, sums of d
+    EP_PLAIN,    // Cf = v
+};
 
 struct GemmArgs {
     const __nv_bfloat16 *A;
@@ -39,233 +59,310 @@ struct GemmArgs {
     const __nv_bfloat16 *B;
     int64_t ldb;
     int64_t M;
-    int N;
+    int N;                  // multiple of 32, at most 256
     int64_t K;              // multiple of 64
-    const float *bias;      // [N] or null
-    float *Cf;              // FP32 output (pre-activation), [M][ldc], or null
-    int64_t ldc;
-    __nv_bfloat16 *H;       // BF16 output (activation), [M][ldh], or null
-    int64_t ldh;
-    __nv_bfloat16 *HT;      // BF16 transposed output, [N][ldt], or null
+    const float *bias;      // [N]
+    float *Cf;              // FP32 output, [M][N], or null
+    __nv_bfloat16 *H;       // BF16 output, [M][N], or null
+    __nv_bfloat16 *HT;      // its transpose, [N][ldt], zero in columns M .. M rounded up to 64, or null
     int64_t ldt;
-    int act;                // 0 none, 1 SiLU
+    const float *X;         // T [M][N] (EP_OUT), Z [M][N] (EP_BACK)
+    float scale;            // EP_OUT
+    float *colsum;          // [tiles][ldsum]: column sums of d over each tile's rows, or null
+    int64_t ldsum;
+    double *loss;           // [tiles]: sum of r^2 (EP_OUT)
+    int act;                // EP_FORWARD: 0 none, 1 SiLU
     int *status;
-    int vec;                // set by gemm(): Cf and H rows take 16-byte vector stores
 };
 
 __device__ inline float silu(float x) { return x / (1.0f + __expf(-x)); }
 
-__global__ void __launch_bounds__(GT) k_gemm(const GemmArgs g)
+// Sums over the warp's lanes of 16 values each by reduce-scatter: lanes 2c and
+// 2c + 1 end with the sum of value c.
+__device__ inline float warp_colsum16(const float (&d)[16], int lane)
+{
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = d[i];
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        const int off = 16 >> s, half = 8 >> s;
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < half; i++) {
+            const float send = up ? v[i] : v[half + i], keep = up ? v[half + i] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Rows m0 .. m0 + 127 of C over the K chunks [k0, k1).
+template <int EP> __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int64_t m0, int k0, int k1, int tile)
 {
     extern __shared__ unsigned char sraw[];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bar[NSTAGE];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ float csum[4][256];
+    __shared__ double lsum[GT / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // operand tiles must start on 1024-byte boundaries (swizzle atoms)
-    const uint32_t raw = smem_u32(sraw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    unsigned char *sbase = sraw + (base - raw);
-    const uint32_t stage_b = (uint32_t)g.N * 128u;
-    const uint32_t stage = STAGE_A + stage_b;
-    const int64_t m0 = (int64_t)blockIdx.x * 128;
+    const uint32_t base = (smem_u32(sraw) + 1023u) & ~1023u;
     const uint32_t ncols = g.N <= 32 ? 32u : g.N <= 64 ? 64u : g.N <= 128 ? 128u : 256u;
     const uint32_t idesc = idesc_bf16(128, g.N);
-
     if (warp == 0) tmem_alloc(&tmem_slot, ncols);
     if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        abort_flag = 0;
+        for (int s = 0; s < NSTAGE; s++) mbar_init(&bar[s], 1);
         mbar_fence_init();
     }
+    const int nk = k1 - k0;
+    auto load = [&](int c) {
+        if (c < nk) {
+            const uint32_t sa = base + (uint32_t)(c % NSTAGE) * STAGE_BYTES, sb = sa + STAGE_A;
+            const int64_t kk = (int64_t)(k0 + c) * 64;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const int r = (i * GT + tid) >> 3, q = tid & 7;
+                const bool on = m0 + r < g.M;
+                cp_async16_zfill(sa + sw128_offset(r, q), g.A + (on ? m0 + r : 0) * g.lda + kk + q * 8, on ? 16u : 0u);
+            }
+            for (int i = tid; i < g.N * 8; i += GT)
+                cp_async16_zfill(sb + sw128_offset(i >> 3, i & 7), g.B + (int64_t)(i >> 3) * g.ldb + kk + (i & 7) * 8, 16u);
+        }
+        cp_async_commit();
+    };
+    for (int c = 0; c < NSTAGE - 1; c++) load(c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    const int64_t nk = g.K / 64;
-
-    for (int64_t kc = 0; kc < nk; kc++) {
-        const int s = (int)(kc & 1);
-        // the MMAs of chunk kc-2 read this stage
-        if (kc >= 2 && !mbar_wait(&bar[s], (uint32_t)((kc - 2) >> 1) & 1u)) abort_flag = 1;
-        __syncthreads();
-        if (abort_flag) break;
-        unsigned char *sa = sbase + (size_t)s * stage;
-        unsigned char *sb = sa + STAGE_A;
-        for (int i = tid; i < 128 * 8; i += GT) {
-            const int r = i >> 3, c = i & 7;
-            const int64_t row = m0 + r;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (row < g.M) v = *reinterpret_cast<const uint4 *>(g.A + row * g.lda + kc * 64 + c * 8);
-            *reinterpret_cast<uint4 *>(sa + sw128_offset(r, c)) = v;
-        }
-        for (int i = tid; i < g.N * 8; i += GT) {
-            const int r = i >> 3, c = i & 7;
-            const uint4 v = *reinterpret_cast<const uint4 *>(g.B + (int64_t)r * g.ldb + kc * 64 + c * 8);
-            *reinterpret_cast<uint4 *>(sb + sw128_offset(r, c)) = v;
-        }
+    bool bad = false;
+    for (int c = 0; c < nk && !bad; c++) {
+        // the ring slot of chunk c + NSTAGE - 1 was read by the MMAs of chunk c - 1
+        bool late = false;
+        if (c >= 1 && c + NSTAGE - 1 < nk) late = !mbar_wait(&bar[(c - 1) % NSTAGE], (uint32_t)((c - 1) / NSTAGE) & 1u);
+        cp_async_wait<NSTAGE - 2>();
         fence_proxy_async();
-        __syncthreads();
+        bad = __syncthreads_or(late);
+        if (bad) break;
         if (tid == 0) {
             tc_fence_after();
-            const uint32_t a_addr = base + (uint32_t)s * stage, b_addr = a_addr + STAGE_A;
+            const uint32_t a = base + (uint32_t)(c % NSTAGE) * STAGE_BYTES, b = a + STAGE_A;
 #pragma unroll
             for (int ks = 0; ks < 4; ks++)
-                tc_mma_bf16(tmem, sw128_desc(a_addr + ks * 32), sw128_desc(b_addr + ks * 32), idesc,
-                            kc > 0 || ks > 0);
-            tc_commit(&bar[s]);
+                tc_mma_bf16(tmem, sw128_desc(a + ks * 32), sw128_desc(b + ks * 32), idesc, c > 0 || ks > 0);
+            tc_commit(&bar[c % NSTAGE]);
         }
+        load(c + NSTAGE - 1);
     }
-    if (!abort_flag && nk > 0) {
-        const int64_t last = nk - 1;
-        if (!mbar_wait(&bar[last & 1], (uint32_t)(last >> 1) & 1u)) abort_flag = 1;
-    }
+    cp_async_wait_all();
+    bool late = false;
+    if (!bad) late = !mbar_wait(&bar[(nk - 1) % NSTAGE], (uint32_t)((nk - 1) / NSTAGE) & 1u);
+    bad = __syncthreads_or(late || bad);
     tc_fence_after();
-    __syncthreads();
-    if (!abort_flag) {
-        const int64_t row = m0 + 32 * warp + lane;
-        for (int col = 0; col < g.N; col += 16) {
+    if (bad) {
+        if (tid == 0) atomicOr(g.status, ST_TIMEOUT);
+    } else {
+        // warp w reads lanes 32 (w mod 4) .. + 31 of the accumulator, warps 0-3
+        // the first half of the columns, warps 4-7 the second
+        const int quad = warp & 3;
+        const int64_t row = m0 + 32 * quad + lane, Mt = (g.M + 63) / 64 * 64;
+        const bool on = row < g.M;
+        double acc = 0.0;
+#pragma unroll 1
+        for (int col = (warp >> 2) * (g.N / 2), end = col + g.N / 2; col < end; col += 16) {
             float v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)col, v);
-            if (row < g.M && g.vec) {
-                // the thread's 16 values of its row: contiguous in Cf and H,
-                // so each goes out as 16-byte stores (a column of HT, across
-                // the warp's rows, is contiguous as it is)
-                float z[16];
+            tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)col, v);
+            if constexpr (EP == EP_PLAIN || EP == EP_FORWARD) {
+                if constexpr (EP == EP_FORWARD)
+#pragma unroll
+                    for (int j = 0; j < 16; j++) v[j] += g.bias[col + j];
+                if (g.Cf && on) {
+                    float4 *d = reinterpret_cast<float4 *>(g.Cf + row * g.N + col);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) d[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                }
+                if (EP == EP_FORWARD && g.act)
+#pragma unroll
+                    for (int j = 0; j < 16; j++) v[j] = silu(v[j]);
+            } else {
+                float x[16];
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const float4 t = on ? __ldg(reinterpret_cast<const float4 *>(g.X + row * g.N + col) + q)
+                                        : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    x[4 * q] = t.x;
+                    x[4 * q + 1] = t.y;
+                    x[4 * q + 2] = t.z;
+                    x[4 * q + 3] = t.w;
+                }
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    if constexpr (EP == EP_OUT) {
+                        const float r = (v[j] + g.bias[col + j]) - x[j];
+                        if (on) acc += (double)r * r;
+                        v[j] = g.scale * r;
+                    } else {
+                        const float sg = 1.0f / (1.0f + __expf(-x[j]));
+                        v[j] = v[j] * sg * (1.0f + x[j] * (1.0f - sg));
+                    }
+                    if (!on) v[j] = 0.0f;
+                }
+                const float cs = warp_colsum16(v, lane);
+                if ((lane & 1) == 0) csum[quad][col + (lane >> 1)] = cs;
+            }
+            if constexpr (EP != EP_PLAIN) {
                 uint32_t hp[8];
 #pragma unroll
-                for (int j = 0; j < 16; j++) z[j] = v[j] + (g.bias ? g.bias[col + j] : 0.0f);
-#pragma unroll
                 for (int j = 0; j < 16; j += 2) {
-                    const float h0 = g.act ? silu(z[j]) : z[j], h1 = g.act ? silu(z[j + 1]) : z[j + 1];
-                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(h0, h1);
+                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(on ? v[j] : 0.0f, on ? v[j + 1] : 0.0f);
                     hp[j / 2] = *reinterpret_cast<const uint32_t *>(&p2);
-                    if (g.HT) {
+                    if (g.HT && row < Mt) {
                         g.HT[(int64_t)(col + j) * g.ldt + row] = p2.x;
                         g.HT[(int64_t)(col + j + 1) * g.ldt + row] = p2.y;
                     }
                 }
-                if (g.Cf) {
-                    float4 *d = reinterpret_cast<float4 *>(g.Cf + row * g.ldc + col);
-#pragma unroll
-                    for (int q = 0; q < 4; q++) d[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
-                }
-                if (g.H) {
-                    uint4 *d = reinterpret_cast<uint4 *>(g.H + row * g.ldh + col);
+                if (g.H && on) {
+                    uint4 *d = reinterpret_cast<uint4 *>(g.H + row * g.N + col);
                     d[0] = make_uint4(hp[0], hp[1], hp[2], hp[3]);
                     d[1] = make_uint4(hp[4], hp[5], hp[6], hp[7]);
                 }
-            } else if (row < g.M) {
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    float z = v[j] + (g.bias ? g.bias[col + j] : 0.0f);
-                    if (g.Cf) g.Cf[row * g.ldc + col + j] = z;
-                    const float h = g.act ? silu(z) : z;
-                    const __nv_bfloat16 hb = __float2bfloat16_rn(h);
-                    if (g.H) g.H[row * g.ldh + col + j] = hb;
-                    if (g.HT) g.HT[(int64_t)(col + j) * g.ldt + row] = hb;
-                }
             }
         }
-    } else if (tid == 0) {
-        atomicOr(g.status, ST_TIMEOUT);
+        if constexpr (EP == EP_OUT || EP == EP_BACK) {
+            if (EP == EP_OUT) {
+                acc = warp_allsum(acc);
+                if (lane == 0) lsum[warp] = acc;
+            }
+            __syncthreads();
+            if (tid < g.N) g.colsum[tile * g.ldsum + tid] = (csum[0][tid] + csum[1][tid]) + (csum[2][tid] + csum[3][tid]);
+            if (EP == EP_OUT && tid == 0) {
+                double s = 0.0;
+                for (int w = 0; w < GT / 32; w++) s += lsum[w];
+                g.loss[tile] = s;
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, ncols);
 }
 
-int gemm(const GemmArgs &g0, cudaStream_t s)
+template <int EP> __global__ void __launch_bounds__(GT) k_gemm(const GemmArgs g)
 {
-    GemmArgs g = g0;
-    if (g.M <= 0) return DVM_OK;
-    g.vec = (reinterpret_cast<uintptr_t>(g.Cf) % 16 == 0 && g.ldc % 4 == 0 &&
-             reinterpret_cast<uintptr_t>(g.H) % 16 == 0 && g.ldh % 8 == 0) ? 1 : 0;
-    if (g.K % 64 || g.N % 16 || g.N < 16 || g.N > 256) return DVM_EINVAL;
-    const size_t dyn = 2 * (size_t)(STAGE_A + (uint32_t)g.N * 128u) + 1024;
-    static bool configured = false;
-    if (!configured) {
-        if (cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (16384 + 32768) + 1024) !=
-            cudaSuccess)
-            return DVM_ECUDA;
-        configured = true;
+    gemm_tile<EP>(g, (int64_t)blockIdx.x * 128, 0, (int)(g.K / 64), blockIdx.x);
+}
+
+// Partial weight gradients of all four layers: CTA (tile, split), tiles 0-1,
+// 2-3, 4-5 and 6 the rows of gW1, gW2, gW3 and gW4; part [splits][MLP_NPARAM]
+// in the parameters' order.
+struct WgradArgs {
+    const __nv_bfloat16 *A[4], *B[4];  // dZ^T [out][ld], activation^T [in][ld]
+    int64_t ld;
+    int chunks;                        // of 64 rows of the batch
+    int64_t off[4];
+    float *part;
+    int *status;
+};
+constexpr int WG_TILES = 7;
+
+__global__ void __launch_bounds__(GT) k_wgrad(const WgradArgs a)
+{
+    const int l = blockIdx.x >> 1, per = (a.chunks + gridDim.y - 1) / gridDim.y;
+    const int k0 = blockIdx.y * per, k1 = min(a.chunks, k0 + per);
+    GemmArgs g{};
+    g.A = a.A[l];
+    g.B = a.B[l];
+    g.lda = g.ldb = a.ld;
+    g.M = l == 3 ? 64 : 256;
+    g.N = l == 0 ? 64 : 256;
+    g.Cf = a.part + (int64_t)blockIdx.y * MLP_NPARAM + a.off[l];
+    g.status = a.status;
+    gemm_tile<EP_PLAIN>(g, (int64_t)(blockIdx.x & 1) * 128, k0, k1, 0);
+}
+
+// g = sum over splits of the partial weight gradients, and over tiles of the
+// partial bias gradients; loss = sum over tiles
+struct ReduceArgs {
+    const float *part, *bias;  // [splits][MLP_NPARAM], [tiles][832]
+    const double *lossp;       // [tiles]
+    int splits, tiles;
+    float *g;
+    double *loss;
+};
+__global__ void __launch_bounds__(256) k_grad_reduce(const ReduceArgs r)
+{
+    const int q = blockIdx.x * 256 + threadIdx.x;
+    // the flat order: W1 (16384) b1 (256) W2 (65536) b2 (256) W3 b3 W4 (16384) b4 (64)
+    if (q < MLP_NPARAM) {
+        int b = -1;
+        if (q >= 16384 && q < 16640) b = q - 16384;
+        else if (q >= 82176 && q < 82432) b = 256 + q - 82176;
+        else if (q >= 147968 && q < 148224) b = 512 + q - 147968;
+        else if (q >= 164608) b = 768 + q - 164608;
+        float s = 0.0f;
+        if (b < 0) {
+#pragma unroll 8
+            for (int k = 0; k < r.splits; k++) s += __ldg(r.part + (int64_t)k * MLP_NPARAM + q);
+        } else {
+#pragma unroll 16
+            for (int k = 0; k < r.tiles; k++) s += __ldg(r.bias + (int64_t)k * 832 + b);
+        }
+        r.g[q] = s;
     }
-    k_gemm<<<(unsigned)((g.M + 127) / 128), GT, dyn, s>>>(g);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double s = 0.0;
+        for (int k = threadIdx.x; k < r.tiles; k += 32) s += r.lossp[k];
+        s = warp_allsum(s);
+        if (threadIdx.x == 0) *r.loss = s;
+    }
+}
+
+constexpr size_t GEMM_DYN = (size_t)NSTAGE * STAGE_BYTES + 1024;
+
+template <typename Kern> int gemm_shape(Kern *kern)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_DYN) == cudaSuccess
+               ? DVM_OK
+               : DVM_ECUDA;
+}
+
+template <int EP> int gemm(const GemmArgs &g, cudaStream_t s)
+{
+    if (g.M <= 0) return DVM_OK;
+    if (g.K % 64 || g.K < 64 || g.N % 32 || g.N < 32 || g.N > 256) return DVM_EINVAL;
+    if (gemm_shape(k_gemm<EP>)) return DVM_ECUDA;
+    k_gemm<EP><<<(unsigned)((g.M + 127) / 128), GT, GEMM_DYN, s>>>(g);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
 }
 
 // ---- elementwise kernels ------------------------------------------------------
-__global__ void k_to_bf16(const float *x, __nv_bfloat16 *y, __nv_bfloat16 *yt, int64_t n, int cols, int64_t ldt)
+// 64 rows of x [n][64] to BF16 rows y and, if yt is given, columns of yt
+// [64][ldt] (zero in rows n .. n rounded up to 64)
+__global__ void __launch_bounds__(256) k_to_bf16(const float *x, __nv_bfloat16 *y, __nv_bfloat16 *yt, int64_t n, int64_t ldt)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n * cols; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = q / cols;
-        const int c = (int)(q - r * cols);
-        const __nv_bfloat16 b = __float2bfloat16_rn(x[q]);
-        if (y) y[q] = b;
-        if (yt) yt[(int64_t)c * ldt + r] = b;
+    __shared__ __nv_bfloat16 t[64][66];
+    const int64_t r0 = (int64_t)blockIdx.x * 64;
+    for (int q = threadIdx.x; q < 64 * 16; q += 256) {
+        const int r = q >> 4, c = (q & 15) * 4;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (r0 + r < n) v = __ldg(reinterpret_cast<const float4 *>(x + (r0 + r) * 64 + c));
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        if (r0 + r < n) {
+            uint2 w;
+            w.x = *reinterpret_cast<const uint32_t *>(&a);
+            w.y = *reinterpret_cast<const uint32_t *>(&b);
+            *reinterpret_cast<uint2 *>(y + (r0 + r) * 64 + c) = w;
+        }
+        t[r][c] = a.x;
+        t[r][c + 1] = a.y;
+        t[r][c + 2] = b.x;
+        t[r][c + 3] = b.y;
     }
-}
-
-// dO = 2 (O - T) / (n * 64), accumulate the squared error
-__global__ void k_out_grad(const float *O, const float *T, int64_t n, __nv_bfloat16 *dO, __nv_bfloat16 *dOt,
-                           int64_t ldt, float *dOf, double *loss)
-{
-    __shared__ double red[8];
-    double acc = 0.0;
-    const float scale = 2.0f / ((float)n * 64.0f);
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n * 64; q += (int64_t)gridDim.x * blockDim.x) {
-        const float r = O[q] - T[q];
-        acc += (double)r * r;
-        const float d = scale * r;
-        dOf[q] = d;
-        const __nv_bfloat16 b = __float2bfloat16_rn(d);
-        dO[q] = b;
-        dOt[(q & 63) * ldt + (q >> 6)] = b;
-    }
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    if (!yt) return;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w];
-        atomicAdd(loss, s);
-    }
-}
-
-// dZ = dH * silu'(Z), stored BF16 row-major and transposed
-__global__ void k_silu_grad(const float *dH, const float *Z, int64_t n, int cols, __nv_bfloat16 *dZ,
-                            __nv_bfloat16 *dZt, int64_t ldt, float *dZf)
-{
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n * cols; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = q / cols;
-        const int c = (int)(q - r * cols);
-        const float z = Z[q];
-        const float sg = 1.0f / (1.0f + __expf(-z));
-        const float d = dH[q] * sg * (1.0f + z * (1.0f - sg));
-        dZf[q] = d;
-        const __nv_bfloat16 b = __float2bfloat16_rn(d);
-        dZ[q] = b;
-        dZt[(int64_t)c * ldt + r] = b;
-    }
-}
-
-// column sums of a [n][cols] FP32 matrix into out[cols] (bias gradients)
-__global__ void k_colsum(const float *x, int64_t n, int cols, float *out)
-{
-    const int c = blockIdx.x;
-    float s = 0.0f;
-    for (int64_t r = threadIdx.x; r < n; r += blockDim.x) s += x[r * cols + c];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    __shared__ float red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += red[w];
-        out[c] = t;
-    }
+    for (int q = threadIdx.x; q < 64 * 64; q += 256) yt[(int64_t)(q >> 6) * ldt + r0 + (q & 63)] = t[q & 63][q >> 6];
 }
 
 // FP32 master weights -> BF16 W[out][in] and W^T[in][out]; biases stay FP32
@@ -290,15 +387,6 @@ __global__ void k_adam(float *w, float *m, float *v, const float *g, int64_t n, 
         m[q] = mq;
         v[q] = vq;
         w[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
-    }
-}
-
-// weight gradient of layer l, computed as gW^T for the 64-row layer
-__global__ void k_transpose_f32(const float *x, int rows, int cols, float *y)
-{
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < rows * cols; q += gridDim.x * blockDim.x) {
-        const int r = q / cols, c = q - r * cols;
-        y[c * rows + r] = x[q];
     }
 }
 
@@ -368,6 +456,16 @@ int mlp_cast(Mlp &m, cudaStream_t s)
 
 const float *mlp_bias(const Mlp &m, int l) { return m.w + param_offset(l) + (size_t)L_IN[l] * L_OUT[l]; }
 
+// K splits of the weight gradients: the seven tiles on about all 152 SMs for
+// batches up to 12,000 rows, one chain for larger ones.  The tensor core
+// truncates as it accumulates, so that a chain's sum drifts from the exact one
+// as it grows (relative to the gradient's norm: 1.8e-6 at 3,000 rows, 7e-6 at
+// 8,192, 1.8e-5 at 16,000, 8.5e-5 at 60,000); split sums are the more exact
+// ones, but beyond 12,000 rows they would move a gradient by more than 2e-5
+// from the one-chain value that earlier training runs were made with.  One chain on
+// pipelined loads takes 0.26 ms more at 30,000 rows than 21 splits.
+static int wgrad_splits(int64_t n) { return n <= 12000 ? (int)std::min<int64_t>(21, (n + 63) / 64) : 1; }
+
 // working buffers for a batch of n rows (n padded to a multiple of 64)
 int mlp_reserve(Mlp &m, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree)
 {
@@ -375,79 +473,77 @@ int mlp_reserve(Mlp &m, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree
     if (np <= m.cap) return DVM_OK;
     for (auto &b : m.work) b.reset(dfree);
     m.cap = 0;
-    // X, Xt, Z1-3 (f32), H1-3, H1t-3t, O (f32), T (f32), dO, dOt, dOf, dH (f32), dZ, dZt, dZf
-    const size_t sz[] = {(size_t)np * 64 * 2, (size_t)np * 64 * 2,       // X, Xt
+    const size_t tiles = (size_t)(np + 127) / 128;
+    const size_t sz[] = {(size_t)np * 64 * 2, (size_t)np * 64 * 2,           // X, Xt
                          (size_t)np * 256 * 4 * 3,                           // Z1..Z3
                          (size_t)np * 256 * 2 * 3, (size_t)np * 256 * 2 * 3, // H, Ht
-                         (size_t)np * 64 * 4, (size_t)np * 64 * 4,           // O, T
-                         (size_t)np * 64 * 2, (size_t)np * 64 * 2, (size_t)np * 64 * 4,  // dO, dOt, dOf
-                         (size_t)np * 256 * 4,                               // dH
-                         (size_t)np * 256 * 2, (size_t)np * 256 * 2, (size_t)np * 256 * 4};  // dZ, dZt, dZf
+                         (size_t)np * 64 * 2, (size_t)np * 64 * 2,           // dO, dOt
+                         (size_t)np * 256 * 2 * 2, (size_t)np * 256 * 2 * 3, // dZ (two in turn), dZt of each layer
+                         (size_t)21 * MLP_NPARAM * 4,                        // partial weight gradients (at most 21 splits)
+                         tiles * 832 * 4, tiles * 8};                        // partial bias gradients and losses
     static_assert(sizeof(sz) / sizeof(sz[0]) == MLP_NWORK, "work buffer count");
     for (int i = 0; i < MLP_NWORK; i++) {
         m.work[i].p = alloc(sz[i]);
         m.work[i].bytes = sz[i];
         if (!m.work[i].p) return DVM_ENOMEM;
-        cudaMemset(m.work[i].p, 0, sz[i]);
     }
     m.cap = np;
     return DVM_OK;
 }
 
-// forward on rows X (BF16 [n][64] in work X); with train = true also keeps
-// pre-activations, activations and their transposes for the backward pass
-static int forward(Mlp &m, int64_t n, bool train, int *status, cudaStream_t s)
+// layers 1 to 3 on rows X (BF16 [n][64] in work X); with train = true also
+// keeps pre-activations and transposed activations for the backward pass
+static int forward3(Mlp &m, int64_t n, bool train, int *status, cudaStream_t s)
 {
     const int64_t np = m.cap;
-    auto *X = static_cast<__nv_bfloat16 *>(m.work[W_X].p);
     auto *Z = static_cast<float *>(m.work[W_Z].p);
     auto *H = static_cast<__nv_bfloat16 *>(m.work[W_H].p);
     auto *Ht = static_cast<__nv_bfloat16 *>(m.work[W_HT].p);
-    auto *O = static_cast<float *>(m.work[W_O].p);
-    const __nv_bfloat16 *in = X;
-    int64_t ld_in = 64;
-    for (int l = 0; l < 4; l++) {
+    const __nv_bfloat16 *in = static_cast<__nv_bfloat16 *>(m.work[W_X].p);
+    for (int l = 0; l < 3; l++) {
         GemmArgs g{};
         g.A = in;
-        g.lda = ld_in;
+        g.lda = g.ldb = g.K = L_IN[l];
         g.B = m.W[l];
-        g.ldb = L_IN[l];
         g.M = n;
-        g.N = L_OUT[l];
-        g.K = L_IN[l];
+        g.N = 256;
         g.bias = mlp_bias(m, l);
         g.status = status;
-        if (l < 3) {
-            g.act = 1;
-            g.Cf = train ? Z + (size_t)l * np * 256 : nullptr;
-            g.ldc = 256;
-            g.H = H + (size_t)l * np * 256;
-            g.ldh = 256;
-            g.HT = train ? Ht + (size_t)l * np * 256 : nullptr;
-            g.ldt = np;
-            in = g.H;
-            ld_in = 256;
-        } else {
-            g.act = 0;
-            g.Cf = O;
-            g.ldc = 64;
-        }
-        int rc = gemm(g, s);
+        g.act = 1;
+        g.Cf = train ? Z + (size_t)l * np * 256 : nullptr;
+        g.H = H + (size_t)l * np * 256;
+        g.HT = train ? Ht + (size_t)l * np * 256 : nullptr;
+        g.ldt = np;
+        in = g.H;
+        int rc = gemm<EP_FORWARD>(g, s);
         if (rc) return rc;
     }
     return DVM_OK;
 }
 
+static GemmArgs layer4(Mlp &m, int64_t n, int *status)
+{
+    GemmArgs g{};
+    g.A = static_cast<__nv_bfloat16 *>(m.work[W_H].p) + (size_t)2 * m.cap * 256;
+    g.B = m.W[3];
+    g.lda = g.ldb = g.K = 256;
+    g.M = n;
+    g.N = 64;
+    g.bias = mlp_bias(m, 3);
+    g.status = status;
+    return g;
+}
+
 int mlp_forward(Mlp &m, const float *x_dev, int64_t n, float *y_dev, int *status, cudaStream_t s)
 {
     if (n > m.cap) return DVM_EINVAL;
-    k_to_bf16<<<blocks(n * 64), 256, 0, s>>>(x_dev, static_cast<__nv_bfloat16 *>(m.work[W_X].p), nullptr, n, 64, 0);
+    k_to_bf16<<<(unsigned)((n + 63) / 64), 256, 0, s>>>(x_dev, static_cast<__nv_bfloat16 *>(m.work[W_X].p), nullptr, n, 0);
     count_launch();
-    int rc = forward(m, n, false, status, s);
+    int rc = forward3(m, n, false, status, s);
     if (rc) return rc;
-    return cudaMemcpyAsync(y_dev, m.work[W_O].p, (size_t)n * 64 * 4, cudaMemcpyDeviceToDevice, s) == cudaSuccess
-               ? DVM_OK
-               : DVM_ECUDA;
+    GemmArgs g = layer4(m, n, status);
+    g.Cf = y_dev;
+    return gemm<EP_FORWARD>(g, s);
 }
 
 // loss and gradient (m.g) for rows x_dev / targets t_dev (FP32 [n][64])
@@ -455,80 +551,68 @@ int mlp_grad(Mlp &m, const float *x_dev, const float *t_dev, int64_t n, int *sta
 {
     if (n > m.cap) return DVM_EINVAL;
     const int64_t np = m.cap;
+    const int tiles = (int)((n + 127) / 128), splits = wgrad_splits(n);
     auto *X = static_cast<__nv_bfloat16 *>(m.work[W_X].p);
     auto *Xt = static_cast<__nv_bfloat16 *>(m.work[W_XT].p);
     auto *Z = static_cast<float *>(m.work[W_Z].p);
-    auto *H = static_cast<__nv_bfloat16 *>(m.work[W_H].p);
     auto *Ht = static_cast<__nv_bfloat16 *>(m.work[W_HT].p);
-    auto *O = static_cast<float *>(m.work[W_O].p);
     auto *dO = static_cast<__nv_bfloat16 *>(m.work[W_DO].p);
     auto *dOt = static_cast<__nv_bfloat16 *>(m.work[W_DOT].p);
-    auto *dOf = static_cast<float *>(m.work[W_DOF].p);
-    auto *dH = static_cast<float *>(m.work[W_DH].p);
     auto *dZ = static_cast<__nv_bfloat16 *>(m.work[W_DZ].p);
     auto *dZt = static_cast<__nv_bfloat16 *>(m.work[W_DZT].p);
-    auto *dZf = static_cast<float *>(m.work[W_DZF].p);
-    // the weight gradients sum over K = n rounded up to 64: the transposed
-    // operands must hold zeros past row n
-    const int64_t nk = (n + 63) / 64 * 64;
-    cudaMemsetAsync(Xt, 0, m.work[W_XT].bytes, s);
-    cudaMemsetAsync(Ht, 0, m.work[W_HT].bytes, s);
-    cudaMemsetAsync(dOt, 0, m.work[W_DOT].bytes, s);
-    cudaMemsetAsync(dZt, 0, m.work[W_DZT].bytes, s);
-    k_to_bf16<<<blocks(n * 64), 256, 0, s>>>(x_dev, X, Xt, n, 64, np);
+    auto *bias = static_cast<float *>(m.work[W_BIAS].p);
+    auto *lossp = static_cast<double *>(m.work[W_LOSS].p);
+    k_to_bf16<<<(unsigned)((n + 63) / 64), 256, 0, s>>>(x_dev, X, Xt, n, np);
     count_launch();
-    int rc = forward(m, n, true, status, s);
+    int rc = forward3(m, n, true, status, s);
     if (rc) return rc;
-    cudaMemsetAsync(m.loss, 0, 8, s);
-    k_out_grad<<<blocks(n * 64), 256, 0, s>>>(O, t_dev, n, dO, dOt, np, dOf, m.loss);
-    count_launch();
-    // layer 4: gW4^T[in][out] = H3^T . dO ; gb4 = colsum dO ; dH3 = dO . W4
-    {
-        GemmArgs g{};
-        g.A = Ht + (size_t)2 * np * 256; g.lda = np;
-        g.B = dOt; g.ldb = np;
-        g.M = 256; g.N = 64; g.K = nk;
-        g.Cf = dH; g.ldc = 64;  // scratch for gW4^T
-        g.status = status;
-        if ((rc = gemm(g, s))) return rc;
-        k_transpose_f32<<<blocks(256 * 64), 256, 0, s>>>(dH, 256, 64, m.g + param_offset(3));
-        count_launch();
-        k_colsum<<<64, 256, 0, s>>>(dOf, n, 64, m.g + param_offset(3) + 256 * 64);
-        count_launch();
-        GemmArgs h{};
-        h.A = dO; h.lda = 64;
-        h.B = m.WT[3]; h.ldb = 64;
-        h.M = n; h.N = 256; h.K = 64;
-        h.Cf = dH; h.ldc = 256;
-        h.status = status;
-        if ((rc = gemm(h, s))) return rc;
-    }
+    // dO = 2 (O - T) / (64 n)
+    GemmArgs g = layer4(m, n, status);
+    g.X = t_dev;
+    g.scale = 2.0f / ((float)n * 64.0f);
+    g.H = dO;
+    g.HT = dOt;
+    g.ldt = np;
+    g.colsum = bias + 768;
+    g.ldsum = 832;
+    g.loss = lossp;
+    if ((rc = gemm<EP_OUT>(g, s))) return rc;
+    // dZ_l = (dZ_{l+1} . W_{l+1}) silu'(Z_l)
     for (int l = 2; l >= 0; l--) {
-        // dZ_l = dH_l * silu'(Z_l)
-        k_silu_grad<<<blocks(n * 256), 256, 0, s>>>(dH, Z + (size_t)l * np * 256, n, 256, dZ, dZt, np, dZf);
-        count_launch();
-        // gW_l[out][in] = dZ^T . (input of layer l)
-        GemmArgs g{};
-        g.A = dZt; g.lda = np;
-        g.B = l > 0 ? Ht + (size_t)(l - 1) * np * 256 : Xt; g.ldb = np;
-        g.M = 256; g.N = L_IN[l]; g.K = nk;
-        g.Cf = m.g + param_offset(l); g.ldc = L_IN[l];
-        g.status = status;
-        if ((rc = gemm(g, s))) return rc;
-        k_colsum<<<256, 256, 0, s>>>(dZf, n, 256, m.g + param_offset(l) + (size_t)L_IN[l] * 256);
-        count_launch();
-        if (l > 0) {
-            // dH_{l-1} = dZ_l . W_l
-            GemmArgs h{};
-            h.A = dZ; h.lda = 256;
-            h.B = m.WT[l]; h.ldb = 256;
-            h.M = n; h.N = 256; h.K = 256;
-            h.Cf = dH; h.ldc = 256;
-            h.status = status;
-            if ((rc = gemm(h, s))) return rc;
-        }
+        GemmArgs h{};
+        h.A = l == 2 ? dO : dZ + (size_t)((l + 1) & 1) * np * 256;
+        h.B = m.WT[l + 1];
+        h.lda = h.ldb = h.K = L_OUT[l + 1];
+        h.M = n;
+        h.N = 256;
+        h.X = Z + (size_t)l * np * 256;
+        h.H = l > 0 ? dZ + (size_t)(l & 1) * np * 256 : nullptr;
+        h.HT = dZt + (size_t)l * np * 256;
+        h.ldt = np;
+        h.colsum = bias + 256 * l;
+        h.ldsum = 832;
+        h.status = status;
+        if ((rc = gemm<EP_BACK>(h, s))) return rc;
     }
-    (void)H;
+    // gW_l[out][in] = dZ_l^T . (input of layer l)
+    WgradArgs w{};
+    for (int l = 0; l < 4; l++) {
+        w.A[l] = l < 3 ? dZt + (size_t)l * np * 256 : dOt;
+        w.B[l] = l > 0 ? Ht + (size_t)(l - 1) * np * 256 : Xt;
+        w.off[l] = (int64_t)param_offset(l);
+    }
+    w.ld = np;
+    w.chunks = (int)((n + 63) / 64);
+    w.part = static_cast<float *>(m.work[W_PART].p);
+    w.status = status;
+    // every split holds at least one chunk
+    const int per = (w.chunks + splits - 1) / splits, used = (w.chunks + per - 1) / per;
+    if (gemm_shape(k_wgrad)) return DVM_ECUDA;
+    k_wgrad<<<dim3(WG_TILES, used), GT, GEMM_DYN, s>>>(w);
+    count_launch();
+    const ReduceArgs r{w.part, bias, lossp, used, tiles, m.g, m.loss};
+    k_grad_reduce<<<(unsigned)((MLP_NPARAM + 255) / 256), 256, 0, s>>>(r);
+    count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
 }
 

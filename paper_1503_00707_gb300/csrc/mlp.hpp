@@ -12,7 +12,7 @@ namespace dvm {
 // W2[256][256] b2 W3[256][256] b3 W4[64][256] b4[64] (W[out][in]).
 constexpr int64_t MLP_NPARAM = 164672;
 
-enum { W_X = 0, W_XT, W_Z, W_H, W_HT, W_O, W_T, W_DO, W_DOT, W_DOF, W_DH, W_DZ, W_DZT, W_DZF, MLP_NWORK };
+enum { W_X = 0, W_XT, W_Z, W_H, W_HT, W_DO, W_DOT, W_DZ, W_DZT, W_PART, W_BIAS, W_LOSS, MLP_NWORK };
 
 struct DevBuf {
     void *p = nullptr;
