@@ -586,7 +586,6 @@ void hs_free(HsTables &t, const DevFree &dfree)
     if (t.d_idx) dfree(t.d_idx);
     if (t.d_b) dfree(t.d_b);
     if (t.d_xi) dfree(t.d_xi);
-    if (t.d_jpk) dfree(t.d_jpk);
     if (t.d_tab) dfree(t.d_tab);
     if (t.d_lane) dfree(t.d_lane);
     if (t.d_desc) dfree(t.d_desc);
@@ -600,7 +599,6 @@ void hs_free(HsTables &t, const DevFree &dfree)
     t.d_idx = nullptr;
     t.d_b = nullptr;
     t.d_xi = nullptr;
-    t.d_jpk = nullptr;
     t.d_bc = nullptr;
     t.bc_cells = 0;
     t.ready = false;
@@ -699,17 +697,8 @@ int hs_build(HsTables &t, const int n[3], const double lo[3], const double h[3],
         }
     }
     std::vector<float> xf(3 * (size_t)nv);
-    std::vector<uint32_t> jp((size_t)nv);
-    for (int v = 0; v < nv; v++) {
-        uint32_t w = 0;
-        for (int d = 0; d < 3; d++) {
-            xf[(size_t)d * nv + v] = (float)xi[3 * (size_t)v + d];
-            // node k of axis d: xi = lo + (k + 1/2) h = (h/2) (2k + 1 - n)
-            const int k = (int)std::lround((xi[3 * (size_t)v + d] - lo[d]) / h[d] - 0.5);
-            w |= (uint32_t)(2 * k + 1 - n[d] + 64) << (8 * d);
-        }
-        jp[v] = w;
-    }
+    for (int v = 0; v < nv; v++)
+        for (int d = 0; d < 3; d++) xf[(size_t)d * nv + v] = (float)xi[3 * (size_t)v + d];
     t.hh = 0.5 * h[0];
     for (int d = 0; d < 3; d++) t.half[d] = n[d] / 2;
     // the device's copy of a table
@@ -720,7 +709,6 @@ int hs_build(HsTables &t, const int n[3], const double lo[3], const double h[3],
         return cudaMemcpy(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess ? DVM_OK : DVM_ECUDA;
     };
     int rc = put(t.d_xi, xf);
-    if (!rc) rc = put(t.d_jpk, jp);
     if (nv <= HS_PAIR_MAX_NV) {
         HsPacked pk;
         hs_pack(t.host_idx, t.host_b, nv, trials, pk);

@@ -29,7 +29,6 @@ struct HsTables {
     uint32_t *d_idx = nullptr;
     float *d_b = nullptr;
     float *d_xi = nullptr;            // node velocities [3][nv], FP32
-    uint32_t *d_jpk = nullptr;        // per node: xi_d = hh j_d, j_d odd, packed as bytes j_d + 64
     double hh = 0.0;                  // half the velocity spacing (the same on every axis)
     int half[3] = {0, 0, 0};          // nodes per axis / 2 (the grid's sign-group shape)
     // scratch for bc_cells cells at a time: B and C, [2][bc_cells][nv], and f

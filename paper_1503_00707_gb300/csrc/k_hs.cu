@@ -32,6 +32,7 @@
 #include "async.cuh"
 #include "common.cuh"
 #include "hs.hpp"
+#include "quads.cuh"
 
 namespace dvm {
 
@@ -41,7 +42,7 @@ namespace {
 
 constexpr int HE = 32;    // trials held per thread of k_hs_bc
 constexpr int HT = 512;   // threads per CTA of k_hs_bc
-constexpr int CT = 256;   // threads per CTA of k_hs_corr
+constexpr int CT = 128;   // threads per CTA of k_hs_corr (at most)
 
 // The rows of a batch: rows r0, r0 + 1, .. (at most nb) of the cells, or of
 // a device list of cells.
@@ -330,36 +331,76 @@ __device__ inline void acc2_prod(Acc2 &a, float x, float xl, float k)
 
 constexpr int NSUM = 20;  // 15 distinct entries of the moment matrix, 5 gain moments
 
+// The signed sums over the eight sign groups that the moment system needs, per
+// position (packed pairs of z nodes), from the sums p and differences m of the
+// groups' pairs along z: S, X, Y, Z as group_sums, and XY = sum s_x s_y x, XZ,
+// YZ.
+__device__ inline void group_sums7(const float2 (&p)[4], const float2 (&m)[4], float2 (&v)[7])
+{
+    const float2 pp0 = f2_add(p[0], p[1]), pm0 = f2_sub(p[1], p[0]);
+    const float2 pp1 = f2_add(p[2], p[3]), pm1 = f2_sub(p[3], p[2]);
+    v[0] = f2_add(pp0, pp1);
+    v[1] = f2_sub(pp1, pp0);
+    v[2] = f2_add(pm0, pm1);
+    v[4] = f2_sub(pm1, pm0);
+    const float2 mp0 = f2_add(m[0], m[1]), mm0 = f2_sub(m[1], m[0]);
+    const float2 mp1 = f2_add(m[2], m[3]), mm1 = f2_sub(m[3], m[2]);
+    v[3] = f2_add(mp0, mp1);
+    v[5] = f2_sub(mp1, mp0);
+    v[6] = f2_add(mm0, mm1);
+}
+
+// sigma = 2^k > 16 max |x|: the split x = q + r against it, q = fl(fl(x +
+// sigma) - sigma), leaves q a multiple of 2^(k-24) whose signed sums over
+// eight groups are exact in FP32, and |r| <= 2^(k-24)
+__device__ inline float2 split_sigma(const float2 (&x)[8])
+{
+    uint32_t mx = 0;
+#pragma unroll
+    for (int o = 0; o < 8; o++)
+        mx = max(mx, max(__float_as_uint(x[o].x) & 0x7fffffffu, __float_as_uint(x[o].y) & 0x7fffffffu));
+    const int ex = min((int)(mx >> 23), 249);
+    const float sg = __int_as_float((ex + 5) << 23);
+    return make_float2(sg, sg);
+}
+
 // k_hs_corr: one CTA per cell.  The correction polynomial of Eq. 6,
 // P = 1 + d.phi, phi = (1, c, |c|^2 - 3), c = (xi - u)/sqrt(T), makes
-// I = C - f P B conserve mass, momentum and energy.  The system is formed
-// exactly: with xi_d = (h/2) j_d (j_d odd integers, the same h on every
-// axis) the integer basis psi^ = (1, j_x, j_y, j_z, |j|^2) spans the same
-// polynomials, so the 15 sums A^_rs = sum_i psi^_r psi^_s f_i B_i and the 5
-// sums c^_r = sum_i psi^_r C_i have integer weights below 2^24 and products
-// split exactly (FMA); Sum2 carries them to double-float, and one thread
-// solves A^ e = c^, e = (1, 0, 0, 0, 0) + L^T d (L the map psi^ -> phi), in
-// FP64: the factor of L A^ L^T (well conditioned), refined twice against the
-// residual of the exact sums.  That residual, sum_i psi_r I_i dV with
-// psi = (1, xi, |xi|^2), goes to res (may be null).  Then I_i is evaluated
-// in FP32 with the FP32 copy of d and f <- f + dt/Kn I (or I to q_out).
-// three CTAs per SM (80 registers): other cells' sums overlap one CTA's
-// serial solve (C4: 7.56 -> 7.29 ms per step; two or four CTAs were slower on
-// one of the 16^3 and 24^3 grids)
-__global__ void __launch_bounds__(CT, 3)
+// I = C - f P B conserve mass, momentum and energy.  With xi_d = (h/2) j_d
+// (j_d odd integers, the same h on every axis) the integer basis psi^ = (1,
+// j_x, j_y, j_z, |j|^2) spans the same polynomials, so the 15 sums A^_rs =
+// sum_i psi^_r psi^_s f_i B_i and the 5 sums c^_r = sum_i psi^_r C_i have
+// integer weights below 2^24.  A thread takes two z nodes at one position of
+// all eight sign groups: f B (its product split exactly) and C, split
+// against the 16 values' largest, give the signed sums over the groups as an
+// exact part and a rest of 2^-19 of it, and 20 products of those by integers,
+// split exactly (FMA), go into Sum2 accumulators: 22 operations a node where a
+// node at a time takes 72.  One thread solves A^ e = c^, e = (1, 0, 0, 0, 0) +
+// L^T d (L the map psi^ -> phi), in FP64: the factor of L A^ L^T (well
+// conditioned), refined twice against the residual of the sums.  That
+// residual, sum_i psi_r I_i dV with psi = (1, xi, |xi|^2), goes to res (may be
+// null).  Then I_i is evaluated in FP32 with the FP32 copy of d and
+// f <- f + dt/Kn I (or I to q_out).
+// Bound by HBM at best (f, B, C in, f out); 12,016 cells x 24^3 (2.66 GB):
+// 1.81 -> 0.87 ms, 16,584 x 16^3 0.94 -> 0.53 ms (a node at a time, FP64 factor,
+// 256 threads before); what is left is the serial solve and the sums' reduction
+// per cell.
+// five CTAs of 128 threads per SM (96 registers): four other cells' passes
+// overlap one cell's serial solve (whole steps at 16^3 / 24^3: 3.53 / 7.80 ms;
+// 6 x 128 3.56 / 8.00, 12 x 64 3.59 / 8.05, 3 x 256 3.74 / 7.93)
+__global__ void __launch_bounds__(CT, 5)
     k_hs_corr(float *__restrict__ f, const float *__restrict__ Bp, const float *__restrict__ Cp,
-              const float *__restrict__ xi3,
-              const uint32_t *__restrict__ jpk, double hh, double dV, const double *__restrict__ mom, int nv,
-              int3 half, float dtkn, Rows rw, float *__restrict__ q_out, double *__restrict__ res, int *status)
+              const float *__restrict__ xi3, double hh, double dV, const double *__restrict__ mom, int nv, int3 half,
+              float dtkn, Rows rw, float *__restrict__ q_out, double *__restrict__ res, int *status)
 {
     __shared__ ffn part[NSUM][CT];
-    __shared__ double S[NSUM];
+    __shared__ double S[NSUM], Lm[25];
     __shared__ float sd[5];
     // row blockIdx.x of B and C belongs to this cell (an entry of the list, if any)
     const int64_t row = blockIdx.x;
     if (row >= rw.count()) return;
     const int64_t cell = rw.cell(row);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x;
     const double *mo = mom + cell * 5;
     const double rho = mo[0], Td = mo[4];
     if (!(rho > 0.0) || !(Td > 0.0) || !isfinite(rho + Td + mo[1] + mo[2] + mo[3])) {
@@ -371,74 +412,91 @@ __global__ void __launch_bounds__(CT, 3)
         }
         return;
     }
+    const int P = nv / 8, hz = half.z;
     float *fc = f + cell * (int64_t)nv;
     const float *Bc = Bp + row * (int64_t)nv, *Cc = Cp + row * (int64_t)nv;
-    // The sums over the nodes, pencil by pencil: a pencil is the line of nodes
-    // along z at fixed (x, y) node indices, both z signs (sign groups 2 o_xy
-    // and 2 o_xy + 1, positions pos .. pos + hz - 1 in each).  Along a pencil
-    // j_x = a and j_y = b are fixed, so with W_k = sum f B j_z^k (k <= 4) and
-    // C_k = sum C j_z^k (k <= 2), s2 = a^2 + b^2, every sum of the system is a
-    // combination of the pencil sums with integer coefficients, e.g.
-    //   sum f B |j|^2 = s2 W_0 + W_2,  sum f B |j|^4 = s2^2 W_0 + 2 s2 W_2 + W_4.
-    // Products by integers below 2^24 split exactly (FMA), so the sums stay
-    // Sum2-exact, at 8 accumulations per node and 27 per pencil instead of
-    // 20 per node.  The entries are numbered as the upper triangle of the 5x5
-    // matrix over (1, j_x, j_y, j_z, |j|^2), then the 5 right-hand sums.
+    auto ld2 = [](const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); };
+    // The entries are numbered as the upper triangle of the 5x5 matrix over
+    // (1, j_x, j_y, j_z, |j|^2), then the 5 right-hand sums.
     Acc2 acc[NSUM];
 #pragma unroll
     for (int k = 0; k < NSUM; k++) acc[k] = Acc2{0.0f, 0.0f};
-    const int hxy = half.x * half.y, P = hxy * half.z, npen = 4 * hxy;
-    for (int pen = tid; pen < npen; pen += CT) {
-        const int oxy = pen / hxy, pos = (pen - oxy * hxy) * half.z;
-        const uint32_t jp0 = jpk[2 * oxy * P + pos];
-        const float a = (float)((int)(jp0 & 0xffu) - 64), b = (float)((int)((jp0 >> 8) & 0xffu) - 64);
-        Acc2 W[5], Cs[3];
+#pragma unroll 1
+    for (int p = 2 * tid; p < P; p += 2 * T) {
+        const int t = p / hz;
+        const float a = (float)(2 * (t / half.y) + 1), b = (float)(2 * (t % half.y) + 1);
+        const float c0 = (float)(2 * (p - t * hz) + 1);
+        float2 w[8], wl[8], V[7], Vr[7];
 #pragma unroll
-        for (int k = 0; k < 5; k++) W[k] = Acc2{0.0f, 0.0f};
-#pragma unroll
-        for (int k = 0; k < 3; k++) Cs[k] = Acc2{0.0f, 0.0f};
-#pragma unroll
-        for (int oz = 0; oz < 2; oz++) {
-            const int v0 = (2 * oxy + oz) * P + pos;
-            for (int m = 0; m < half.z; m++) {
-                const int v = v0 + m;
-                const float fv = fc[v];
-                const float2 q = make_float2(Bc[v], Cc[v]);
-                const float jz = (float)((int)((jpk[v] >> 16) & 0xffu) - 64);
-                const float jz2 = jz * jz;
-                const float w = fv * q.x, wl = fmaf(fv, q.x, -w);  // f B = w + wl exactly
-                acc2_prod(W[0], w, wl, 1.0f);
-                acc2_prod(W[1], w, wl, jz);
-                acc2_prod(W[2], w, wl, jz2);
-                acc2_prod(W[3], w, wl, jz2 * jz);
-                acc2_prod(W[4], w, wl, jz2 * jz2);
-                acc2_prod(Cs[0], q.y, 0.0f, 1.0f);
-                acc2_prod(Cs[1], q.y, 0.0f, jz);
-                acc2_prod(Cs[2], q.y, 0.0f, jz2);
-            }
+        for (int o = 0; o < 8; o++) {
+            w[o] = *reinterpret_cast<const float2 *>(fc + o * P + p);
+            wl[o] = ld2(Bc + o * P + p);
         }
-        const float s2 = a * a + b * b;
-        auto put = [&](int k, const Acc2 &x, float coef) { acc2_prod(acc[k], x.s, x.e, coef); };
-        put(0, W[0], 1.0f);                                         // (1, 1)
-        put(1, W[0], a);                                            // (1, j_x)
-        put(2, W[0], b);                                            // (1, j_y)
-        put(3, W[1], 1.0f);                                         // (1, j_z)
-        put(4, W[0], s2); put(4, W[2], 1.0f);                       // (1, |j|^2)
-        put(5, W[0], a * a);                                        // (j_x, j_x)
-        put(6, W[0], a * b);                                        // (j_x, j_y)
-        put(7, W[1], a);                                            // (j_x, j_z)
-        put(8, W[0], a * s2); put(8, W[2], a);                      // (j_x, |j|^2)
-        put(9, W[0], b * b);                                        // (j_y, j_y)
-        put(10, W[1], b);                                           // (j_y, j_z)
-        put(11, W[0], b * s2); put(11, W[2], b);                    // (j_y, |j|^2)
-        put(12, W[2], 1.0f);                                        // (j_z, j_z)
-        put(13, W[1], s2); put(13, W[3], 1.0f);                     // (j_z, |j|^2)
-        put(14, W[0], s2 * s2); put(14, W[2], 2.0f * s2); put(14, W[4], 1.0f);  // (|j|^2, |j|^2)
-        put(15, Cs[0], 1.0f);
-        put(16, Cs[0], a);
-        put(17, Cs[0], b);
-        put(18, Cs[1], 1.0f);
-        put(19, Cs[0], s2); put(19, Cs[2], 1.0f);
+#pragma unroll
+        for (int o = 0; o < 8; o++) {
+            // f B = w + wl exactly
+            const float2 m = __fmul2_rn(w[o], wl[o]);
+            wl[o] = __ffma2_rn(w[o], wl[o], make_float2(-m.x, -m.y));
+            w[o] = m;
+        }
+        // the sums of x + xl over the groups: exact part to V, rest to Vr
+        auto sums = [&](const float2 (&x)[8], const float2 *xl) {
+            const float2 sg = split_sigma(x);
+            float2 qp[4], qm[4], rp[4], rm[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const float2 q0 = f2_sub(f2_add(x[2 * k], sg), sg), q1 = f2_sub(f2_add(x[2 * k + 1], sg), sg);
+                float2 r0 = f2_sub(x[2 * k], q0), r1 = f2_sub(x[2 * k + 1], q1);
+                if (xl) {
+                    r0 = f2_add(r0, xl[2 * k]);
+                    r1 = f2_add(r1, xl[2 * k + 1]);
+                }
+                qp[k] = f2_add(q0, q1);
+                qm[k] = f2_sub(q1, q0);
+                rp[k] = f2_add(r0, r1);
+                rm[k] = f2_sub(r1, r0);
+            }
+            group_sums7(qp, qm, V);
+            group_sums7(rp, rm, Vr);
+        };
+        sums(w, wl);
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const float cz = c0 + 2.0f * e, j2 = a * a + b * b + cz * cz;
+            auto put = [&](int k, int v, float coef) {
+                acc2_prod(acc[k], e ? V[v].y : V[v].x, e ? Vr[v].y : Vr[v].x, coef);
+            };
+            put(0, 0, 1.0f);          // (1, 1)
+            put(1, 1, a);             // (1, j_x)
+            put(2, 2, b);             // (1, j_y)
+            put(3, 3, cz);            // (1, j_z)
+            put(4, 0, j2);            // (1, |j|^2)
+            put(5, 0, a * a);         // (j_x, j_x)
+            put(6, 4, a * b);         // (j_x, j_y)
+            put(7, 5, a * cz);        // (j_x, j_z)
+            put(8, 1, a * j2);        // (j_x, |j|^2)
+            put(9, 0, b * b);         // (j_y, j_y)
+            put(10, 6, b * cz);       // (j_y, j_z)
+            put(11, 2, b * j2);       // (j_y, |j|^2)
+            put(12, 0, cz * cz);      // (j_z, j_z)
+            put(13, 3, cz * j2);      // (j_z, |j|^2)
+            put(14, 0, j2 * j2);      // (|j|^2, |j|^2)
+        }
+#pragma unroll
+        for (int o = 0; o < 8; o++) w[o] = ld2(Cc + o * P + p);
+        sums(w, nullptr);
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const float cz = c0 + 2.0f * e, j2 = a * a + b * b + cz * cz;
+            auto put = [&](int k, int v, float coef) {
+                acc2_prod(acc[k], e ? V[v].y : V[v].x, e ? Vr[v].y : Vr[v].x, coef);
+            };
+            put(15, 0, 1.0f);
+            put(16, 1, a);
+            put(17, 2, b);
+            put(18, 3, cz);
+            put(19, 0, j2);
+        }
     }
 #pragma unroll
     for (int k = 0; k < NSUM; k++) {
@@ -447,11 +505,11 @@ __global__ void __launch_bounds__(CT, 3)
         part[k][tid] = ffn{s, (acc[k].s - (s - bb)) + (acc[k].e - bb)};
     }
     __syncthreads();
-    // warp w adds sums w, w + 8, w + 16 over the CTA in double-float
-    for (int k = warp; k < NSUM; k += CT / 32) {
+    // the warps take the sums in turn and add each over the CTA in double-float
+    for (int k = warp; k < NSUM; k += T / 32) {
         ffn a = part[k][lane];
-#pragma unroll
-        for (int t = lane + 32; t < CT; t += 32) a = a + part[k][t];
+#pragma unroll 4
+        for (int t = lane + 32; t < T; t += 32) a = a + part[k][t];
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1)
             a = a + ffn{__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
@@ -459,81 +517,106 @@ __global__ void __launch_bounds__(CT, 3)
     }
     __syncthreads();
     if (warp == 0) {
-        // The 5x5 solve on the lanes of warp 0, in FP64.  phi = L psi^ with
+        // The 5x5 solve on the lanes of warp 0.  phi = L psi^ with
         //   phi_0 = 1, phi_d = be_d + al j_d, phi_4 = |be|^2 - 3 + 2 al be.j + al^2 |j|^2,
         // al = (h/2)/sqrt(T), be = -u/sqrt(T); the system A^ e = c^ with
         // e = (1, 0, 0, 0, 0) + L^T d is factored through the well-conditioned
-        // centred-basis matrix L A^ L^T (an LDL^T on lane 0) and refined twice
-        // against the residual of the exact sums.  Lane 5 r + s holds entry
-        // (r, s) of the 5x5 products; lanes 0..4 hold the vectors.
+        // centred-basis matrix L A^ L^T (an LDL^T on lane 0) and refined
+        // against the FP64 residual of the exact sums.  The factor is FP32
+        // with four rounds (each gains at least three digits; FP64 runs at
+        // 1/64 of the FP32 rate, and an FP64 factor with two rounds took a
+        // third of this kernel's time at 16^3); where it does not converge
+        // to 1e-12, or a pivot fails, the FP64 factor follows.  Lane 5 r + s
+        // holds entry (r, s) of the 5x5 products; lanes 0..4 hold the vectors.
         const double isT = 1.0 / sqrt(Td), al = hh * isT;
-        const double be0 = -mo[1] * isT, be1 = -mo[2] * isT, be2 = -mo[3] * isT;
-        auto Lm = [&](int r, int k) -> double {
-            if (r == 0) return k == 0 ? 1.0 : 0.0;
-            if (r < 4) {
-                const double b = r == 1 ? be0 : (r == 2 ? be1 : be2);
-                return k == 0 ? b : (k == r ? al : 0.0);
-            }
-            if (k == 0) return be0 * be0 + be1 * be1 + be2 * be2 - 3.0;
-            if (k < 4) return 2.0 * al * (k == 1 ? be0 : (k == 2 ? be1 : be2));
-            return al * al;
-        };
+        if (lane < 25) {
+            const int r = lane / 5, k = lane % 5;
+            const double be0 = -mo[1] * isT, be1 = -mo[2] * isT, be2 = -mo[3] * isT;
+            const double bk = k == 1 ? be0 : (k == 2 ? be1 : be2), br = r == 1 ? be0 : (r == 2 ? be1 : be2);
+            double v = r == k ? (r == 0 ? 1.0 : al) : 0.0;
+            if (r >= 1 && r < 4 && k == 0) v = br;
+            if (r == 4) v = k == 0 ? be0 * be0 + be1 * be1 + be2 * be2 - 3.0 : (k < 4 ? 2.0 * al * bk : al * al);
+            Lm[lane] = v;
+        }
+        __syncwarp();
         // entry (r, s) of A^ (index of the upper-triangle sum)
         auto Aj = [&](int r, int q) -> double {
             const int lo = r < q ? r : q, hi = r < q ? q : r;
             return S[lo * 5 - (lo * (lo - 1)) / 2 + (hi - lo)];
         };
-        auto bcast = [](double v, int src) -> double { return __shfl_sync(0xffffffffu, v, src); };
+        auto bcast = [](auto v, int src) { return __shfl_sync(0xffffffffu, v, src); };
         const int r5 = lane < 25 ? lane / 5 : 0, s5 = lane < 25 ? lane % 5 : 0;
         // T1 = L A^ (lane 5 r + s), then Ap = T1 L^T
         double t1 = 0.0;
 #pragma unroll
-        for (int k = 0; k < 5; k++) t1 = fma(Lm(r5, k), Aj(k, s5), t1);
+        for (int k = 0; k < 5; k++) t1 = fma(Lm[r5 * 5 + k], Aj(k, s5), t1);
         double ap = 0.0;
 #pragma unroll
-        for (int k = 0; k < 5; k++) ap = fma(bcast(t1, r5 * 5 + k), Lm(s5, k), ap);
-        double Ap[25];
-#pragma unroll
-        for (int k = 0; k < 25; k++) Ap[k] = bcast(ap, k);
-        double Lf[5][5], Di[5];
-        bool ok = true;
-        if (lane == 0) ok = ldl5<double>(Ap, Lf, Di);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        // lane r < 5: d_r; every lane: the whole d after each broadcast
-        double d[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, R = 0.0;
+        for (int k = 0; k < 5; k++) ap = fma(bcast(t1, r5 * 5 + k), Lm[s5 * 5 + k], ap);
         const int rv = lane < 5 ? lane : 0;
-        for (int it = 0; it < 3; it++) {
-            // e_s = (s == 0) + sum_k L_ks d_k on lane s, then R_r = c^_r - sum_s A^_rs e_s
+        double Arow[5], Lrow[5], Lcol[5];  // row rv of A^ and of L, column rv of L
+#pragma unroll
+        for (int k = 0; k < 5; k++) {
+            Arow[k] = Aj(rv, k);
+            Lrow[k] = Lm[rv * 5 + k];
+            Lcol[k] = Lm[k * 5 + rv];
+        }
+        double d[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, R = 0.0;  // every lane: d; lane r < 5: the residual's row r
+        // R_r = c^_r - sum_s A^_rs e_s on lane r, e_s = (s == 0) + sum_k L_ks d_k
+        auto residual = [&]() {
             double e = rv == 0 ? 1.0 : 0.0;
 #pragma unroll
-            for (int k = 0; k < 5; k++) e = fma(Lm(k, rv), d[k], e);
-            double ev[5];
-#pragma unroll
-            for (int k = 0; k < 5; k++) ev[k] = bcast(e, k);
+            for (int k = 0; k < 5; k++) e = fma(Lcol[k], d[k], e);
             R = S[15 + rv];
 #pragma unroll
-            for (int q = 0; q < 5; q++) R = fma(-Aj(rv, q), ev[q], R);
-            if (it == 2 || !ok) break;
-            // LR = L R on lane r, then the LDL^T solve on lane 0
-            double Rv[5];
+            for (int q = 0; q < 5; q++) R = fma(-Arow[q], bcast(e, q), R);
+        };
+        // `rounds` solves with a factor of type F, and the residual after them
+        auto solve = [&](auto one, int rounds) -> bool {
+            using F = decltype(one);
+            F Ap[25], Lf[5][5], Di[5];
+            const F av = (F)ap;
 #pragma unroll
-            for (int k = 0; k < 5; k++) Rv[k] = bcast(R, k);
-            double lr = 0.0;
+            for (int k = 0; k < 25; k++) Ap[k] = bcast(av, k);
+            bool ok = true;
+            if (lane == 0) ok = ldl5<F>(Ap, Lf, Di);
+            ok = bcast(ok ? 1 : 0, 0) != 0;
+            bool still = false;  // the last correction still moved d
 #pragma unroll
-            for (int k = 0; k < 5; k++) lr = fma(Lm(rv, k), Rv[k], lr);
-            double LR[5], dl[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            for (int k = 0; k < 5; k++) d[k] = 0.0;
+            residual();
+            for (int it = 0; it < rounds && ok; it++) {
+                // LR = L R on lane r, then the LDL^T solve on lane 0
+                double lr = 0.0;
 #pragma unroll
-            for (int k = 0; k < 5; k++) LR[k] = bcast(lr, k);
-            if (lane == 0) ldl5_solve<double>(Lf, Di, LR, dl);
+                for (int k = 0; k < 5; k++) lr = fma(Lrow[k], bcast(R, k), lr);
+                const F lf = (F)lr;
+                F LR[5], dl[5] = {0, 0, 0, 0, 0};
 #pragma unroll
-            for (int k = 0; k < 5; k++) d[k] += bcast(dl[k], 0);
-        }
+                for (int k = 0; k < 5; k++) LR[k] = bcast(lf, k);
+                if (lane == 0) ldl5_solve<F>(Lf, Di, LR, dl);
+                still = false;
+#pragma unroll
+                for (int k = 0; k < 5; k++) {
+                    const F x = bcast(dl[k], 0);
+                    d[k] += (double)x;
+                    still = still || !(fabsf((float)x) <= 1e-12f * (1.0f + fabsf((float)d[k])));
+                }
+                residual();
+            }
+            return ok && (sizeof(F) == 8 || !still);
+        };
+        bool ok = solve(0.0f, 4);
+        if (!ok) ok = solve(0.0, 2);
         bool fin = ok;
 #pragma unroll
         for (int k = 0; k < 5; k++) fin = fin && isfinite(d[k]);
         if (lane == 0 && !fin) atomicOr(status, ST_SINGULAR);
         if (lane < 5) {
-            sd[lane] = fin ? (float)d[lane] : 0.0f;
+            double dv = d[0];
+#pragma unroll
+            for (int k = 1; k < 5; k++) dv = lane == k ? d[k] : dv;
+            sd[lane] = fin ? (float)dv : 0.0f;
             if (res) {
                 const double sc = lane == 0 ? dV : (lane < 4 ? dV * hh : dV * hh * hh);
                 res[cell * 5 + lane] = fin ? sc * R : 0.0;
@@ -544,16 +627,40 @@ __global__ void __launch_bounds__(CT, 3)
     const float ux = (float)mo[1], uy = (float)mo[2], uz = (float)mo[3];
     const float ist = rsqrtf((float)Td);
     const float d0 = sd[0], dx = sd[1], dy = sd[2], dz = sd[3], d4 = sd[4];
+    // P at node = (1 + d0 - 3 d4) + sum over the axes of c (d_axis + d4 c)
+    auto axis = [&](float x, float u, float da) {
+        const float cc = (x - u) * ist;
+        return cc * fmaf(d4, cc, da);
+    };
+    const float k0 = 1.0f + d0 - 3.0f * d4;
+    float *qc = q_out ? q_out + cell * (int64_t)nv : nullptr;
     float worst = 0.0f;
-    for (int v = tid; v < nv; v += CT) {
-        const float fv = fc[v];
-        const float2 q = make_float2(Bc[v], Cc[v]);
-        const float cx = (xi3[v] - ux) * ist, cy = (xi3[nv + v] - uy) * ist, cz = (xi3[2 * nv + v] - uz) * ist;
-        const float P = 1.0f + d0 + dx * cx + dy * cy + dz * cz + d4 * (cx * cx + cy * cy + cz * cz - 3.0f);
-        const float loss = P * q.x;
-        worst = fmaxf(worst, dtkn * loss);
-        if (q_out) q_out[cell * (int64_t)nv + v] = q.y - fv * loss;  // the term I alone, f kept
-        else fc[v] = fmaf(dtkn, q.y - fv * loss, fv);
+#pragma unroll 1
+    for (int p = 2 * tid; p < P; p += 2 * T) {
+        const int v = 7 * P + p;  // the node with every component positive
+        const float x = xi3[v], y = xi3[nv + v];
+        const float2 z = ld2(xi3 + 2 * nv + v);
+        const float px[2] = {axis(-x, ux, dx), axis(x, ux, dx)}, py[2] = {axis(-y, uy, dy), axis(y, uy, dy)};
+        const float2 pz[2] = {make_float2(axis(-z.x, uz, dz), axis(-z.y, uz, dz)),
+                              make_float2(axis(z.x, uz, dz), axis(z.y, uz, dz))};
+        float2 fv[8], bv[8], cv[8];
+#pragma unroll
+        for (int o = 0; o < 8; o++) {
+            fv[o] = *reinterpret_cast<const float2 *>(fc + o * P + p);
+            bv[o] = ld2(Bc + o * P + p);
+            cv[o] = ld2(Cc + o * P + p);
+        }
+#pragma unroll
+        for (int o = 0; o < 8; o++) {
+            const float kxy = k0 + (px[o >> 2] + py[(o >> 1) & 1]);
+            const float2 loss = __fmul2_rn(f2_add(make_float2(kxy, kxy), pz[o & 1]), bv[o]);
+            worst = fmaxf(worst, dtkn * fmaxf(loss.x, loss.y));
+            const float2 I = __ffma2_rn(make_float2(-fv[o].x, -fv[o].y), loss, cv[o]);
+            if (qc) *reinterpret_cast<float2 *>(qc + o * P + p) = I;  // the term alone, f kept
+            else
+                *reinterpret_cast<float2 *>(fc + o * P + p) =
+                    __ffma2_rn(make_float2(dtkn, dtkn), I, fv[o]);
+        }
     }
     if (worst > 1.0f) atomicOr(status, ST_NUDT);
 }
@@ -686,8 +793,12 @@ static int run_batches(const BcLaunch &L, const HsTables &t, float *f, float *bc
                                               t.d_b, status);
         }
         count_launch();
-        k_hs_corr<<<rows, CT, 0, s>>>(f, Bp, Cp, t.d_xi, t.d_jpk, t.hh, c.dV, c.mom, nv,
-                                      make_int3(t.half[0], t.half[1], t.half[2]), c.dtkn, rw, c.q_out, c.res, status);
+        // pairs of z nodes per sign group over rounds of at most CT threads,
+        // evenly (24^3: 864 on 4 x 224)
+        const int units = nv / 16, rounds = (units + CT - 1) / CT, per = (units + rounds - 1) / rounds;
+        k_hs_corr<<<rows, (per + 31) / 32 * 32, 0, s>>>(f, Bp, Cp, t.d_xi, t.hh, c.dV, c.mom, nv,
+                                                        make_int3(t.half[0], t.half[1], t.half[2]), c.dtkn, rw,
+                                                        c.q_out, c.res, status);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return DVM_ECUDA;
     }
