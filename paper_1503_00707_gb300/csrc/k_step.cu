@@ -21,10 +21,10 @@
 //   phase 1  f*_i = (1 - dt invh sum_d |xi_d,i|) f_i + sum_d dt |xi_d,i| sum_k
 //            w_k src_k,i for cell j on packed FP32 pairs, into registers.  The
 //            inputs of each sign group (the cell's own values and the first
-//            upwind source of each axis, Sec. 3.1 step 4) come from a 4-stage
+//            upwind source of each axis, Sec. 3.1 step 4) come from a
 //            shared-memory ring that every thread fills for its own
-//            positions with cp.async, four groups ahead; further sources
-//            behind coarse-fine faces come from L2.  Per-thread FP32 partials
+//            positions with cp.async, four (BF16: eight) groups ahead; further
+//            sources behind coarse-fine faces come from L2.  Per-thread FP32 partials
 //            of the seven sums sum f, sum j_d f, sum j_d^2 f (xi_d = (h_d/2)
 //            j_d, j_d odd) are reduced per warp.
 //   phase 3  the collision of cell j - 2, whose f* waits in one of two
@@ -36,7 +36,8 @@
 // M~ = M (1 + d.phi) (the correction form of Eq. 6) that make M~ carry the
 // moments of f*; per-axis tables g = exp(-c^2/2), P = d_axis c + d4 c^2)
 // runs while the compute warps transport cells j + 1 and j + 2.  Solver warps
-// also fetch the cells' stencils, four iterations ahead.
+// also fetch the cells' stencils, four iterations ahead, and prefetch the
+// cells' own values (an HBM stream) into L2 with one bulk instruction.
 //
 // Phase 3: f^{n+1} = (1 - nu dt) f* + nu dt M~ with M~ = rho (2 pi T)^(-3/2)
 //   gx gy gz (1 + d0 - 3 d4 + Px + Py + Pz), nu = sqrt(8/pi) rho sqrt(T)/Kn.
@@ -49,6 +50,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "../../include/dvm.h"
 #include "async.cuh"
@@ -68,7 +70,10 @@ namespace {
 constexpr int MAXCW = 14;     // compute warps per CTA (at most)
 constexpr int NAX = 32;       // velocity nodes per axis supported
 constexpr int MAXT = MAXCW * 32 + 64;
-constexpr int NST = 4;        // ring stages (one sign group of one cell each)
+// ring stages (one sign group of one cell each): 4 or 8.  BF16 pieces are half
+// as large, and eight stages, a whole cell ahead, keep as many bytes in flight
+// (24^3 BF16: 4.41 -> 4.39 ms); FP32 at 24^3 has shared memory for four.
+template <typename TS> constexpr int ring_stages() { return sizeof(TS) == 2 ? 8 : 4; }
 constexpr int NSS = 4;        // solver result slots (cell j in slot j % NSS)
 constexpr int NSL = 8;        // ring of per-cell stencil slots (dispatched four iterations ahead)
 
@@ -79,9 +84,12 @@ template <> __device__ inline double tc_exp<double>(double x) { return exp(x); }
 // list of the upwind sources that group o uses along axis d: the minus-side
 // list 2d for a positive velocity component, the plus-side list 2d+1 otherwise
 __host__ __device__ constexpr int list_of(int o, int d) { return 2 * d + (((o >> (2 - d)) & 1) ? 0 : 1); }
-template <int DIM> __host__ __device__ constexpr int lists_of(int o)
+// the entries 4 L + k, k = 1..3, of the lists that group o uses
+template <int DIM> __host__ __device__ constexpr uint32_t entries_of(int o)
 {
-    return (1 << list_of(o, 0)) | (1 << list_of(o, 1)) | (DIM == 3 ? (1 << list_of(o, 2)) : 0);
+    uint32_t m = 0;
+    for (int d = 0; d < DIM; d++) m |= 0xeu << (4 * list_of(o, d));
+    return m;
 }
 
 // coefficient slots written by the solver warp for phase 3:
@@ -103,7 +111,7 @@ template <typename TC> struct CellSlot {
     int32_t src[24];     // per list (axis x side) up to 4 sources: cell | group flip << 28
     TC w[24];            // A_k / V_j
     int cnt[6];
-    int xmask;           // lists with more than one source
+    uint32_t xmask;      // bit 4 L + k: list L has a source k >= 1
     TC invh;
 };
 
@@ -155,7 +163,7 @@ constexpr int BAR_P = 1, BAR_C = 5;
 
 template <typename TS, int DIM> constexpr size_t stage_bytes(int P) { return (size_t)(1 + DIM) * P * sizeof(TS); }
 // dynamic shared memory: the ring and the two f* tiles
-template <typename TS, int DIM> constexpr size_t step_dyn_bytes(int P) { return NST * stage_bytes<TS, DIM>(P) + (size_t)2 * 8 * P * sizeof(TS); }
+template <typename TS, int DIM> constexpr size_t step_dyn_bytes(int P) { return ring_stages<TS>() * stage_bytes<TS, DIM>(P) + (size_t)2 * 8 * P * sizeof(TS); }
 
 // the 16- or 8-byte piece of one thread
 template <typename TS> __device__ inline void cp_piece(TS *dst, const TS *src, uint32_t dep)
@@ -655,14 +663,17 @@ __device__ inline int solve_cell(const StepParams &p, StepSmem<TC> &sm, const Co
 
 // PC: the group size P as a compile-time constant (0: read it from p), so
 // that every group offset of the unrolled loops is an immediate.
+// 16^3 grids (192 threads): 96 registers for three CTAs an SM, six solver and
+// twelve compute warps instead of four and eight (27k cells FP32, four steps:
+// 1.40 -> 1.29 ms).
 template <typename TS, int DIM, int COLL, int PC>
-__global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
+__global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_step(const StepParams p)
 {
     using S = Store<TS>;
     using IO = QIO<TS>;
     using TC = typename S::TC;
     using Q4 = QV<TC>;
-    constexpr int VEC = S::VEC;
+    constexpr int VEC = S::VEC, NST = ring_stages<TS>();
 
     const int P = PC ? PC : p.P;  // velocity nodes per sign group
     const int NV = 8 * P;
@@ -730,13 +741,18 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
                 const int32_t flip = t.first >> 28;
                 sl.sidx[lane] = (t.first & 0x0fffffff) * 8 + ((lane & 1) ? flip : -flip);
             }
-            const unsigned xm = __ballot_sync(0xffffffffu, lane < 6 && t.cnt > 1);
+            const int k = lane & 3, cnt = __shfl_sync(0xffffffffu, t.cnt, lane >> 2);
+            const uint32_t xm = __ballot_sync(0xffffffffu, lane < 24 && k >= 1 && k < cnt);
             if (lane == 0) {
-                sl.xmask = (int)xm;
+                sl.xmask = xm;
                 sl.invh = t.invh;
             }
         }
-        if (lane == 0) sl.cell = t.cell;
+        if (lane == 0) {
+            sl.cell = t.cell;
+            // 24^3 FP32: 4.48 -> 4.41 ms against a prefetch per thread and group
+            if (t.cell >= 0) prefetch_l2_bulk(fin + t.cell * NV, (uint32_t)(NV * sizeof(TS)));
+        }
     };
 
     if (warp == 0) {
@@ -833,11 +849,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
         daz = q_make(t);
     }
 
-    // The chunk indices (units of P values) of the cell whose groups are
-    // being copied: its own group 0 and the first source of each list
-    // (group o adds o).  Each thread reads back only the pieces it copied.
+    // Where the thread's positions of the cell whose groups are being copied
+    // lie: its own group 0 and the first source of each list (group o adds o
+    // P, an immediate where P is a compile-time constant).  Each thread reads
+    // back only the pieces it copied.
     const TS *fin_p0 = fin + p0;
-    int idx_own = 0, idx_l[2 * DIM];
+    const TS *at_own = fin_p0, *at_l[2 * DIM];
     // bit b set: parity b has met an empty slot, so every later slot of that
     // parity is empty (its solver warp has stopped writing slot records)
     int ended = 0;
@@ -846,8 +863,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
         const CellSlot<TC> &sl = sm.slot[k % NSL];
         const long long c = slot_cell(k);
 #pragma unroll
-        for (int L = 0; L < 2 * DIM; L++) idx_l[L] = sl.sidx[L];
-        idx_own = (int)c * 8;
+        for (int L = 0; L < 2 * DIM; L++) at_l[L] = fin_p0 + (int64_t)sl.sidx[L] * P;
+        at_own = fin_p0 + c * NV;
         return c >= 0 && active;
     };
     // group o of the pointed cell into stage st; dep orders the previous
@@ -855,10 +872,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
     auto copy_group = [&](bool on, int o, int st, uint32_t dep) {
         if (on) {
             TS *d = ring + (size_t)st * (1 + DIM) * P + p0;
-            cp_piece(d, fin_p0 + (size_t)(uint32_t)(idx_own + o) * P, dep);
+            cp_piece(d, at_own + o * P, dep);
 #pragma unroll
-            for (int a = 0; a < DIM; a++)
-                cp_piece(d + (1 + a) * P, fin_p0 + (size_t)(uint32_t)(idx_l[list_of(o, a)] + o) * P, dep);
+            for (int a = 0; a < DIM; a++) cp_piece(d + (1 + a) * P, at_l[list_of(o, a)] + o * P, dep);
         }
         cp_async_commit();
     };
@@ -879,11 +895,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
         {
             // ================= phase 1: transport of cell j (an empty slot
             // runs only the copy ring, which brings in the next cell)
-            bool on = point(j);  // groups 4..7 of this cell are copied first
-            // the next cell's own values (an HBM stream) are prefetched into L2
-            // one cell ahead, so that their copies four groups later hit L2
-            const long long nxt = slot_cell(j + 1);
-            const TS *pf = fin_p0 + (size_t)(nxt < 0 ? 0 : nxt) * NV;
+            bool on = NST < 8 && point(j);  // the rest of this cell's groups is copied first
             const TC invh = sl.invh;
             const Q4 cs = q_fma(q_splat(-invh), q_add(q_splat(dax + day), daz), q_splat((TC)1));
             TC aw[4], wz[2];
@@ -891,44 +903,69 @@ __global__ void __launch_bounds__(MAXT, 1) k_step(const StepParams p)
             for (int L = 0; L < 4; L++) aw[L] = (L < 2 ? dax : day) * sl.w[L * 4];
             wz[0] = sl.w[16];
             wz[1] = sl.w[20];
+            const uint32_t xm = sl.xmask;
             const Q4 dz0 = q_mul(daz, q_splat(wz[0])), dz1 = q_mul(daz, q_splat(wz[1]));
-            const int xm = sl.xmask;
+            auto transport = [&](auto more) {
 #pragma unroll
-            for (int o = 0; o < 8; o++) {
-                // this thread's pieces of group o have landed when at most
-                // NST - 1 younger copy groups are pending
-                cp_async_wait<NST - 1>();
-                Q4 fs = q_splat((TC)0);
-                if (valid && active) {
-                    const TS *st = ring + (size_t)(o % NST) * (1 + DIM) * P + p0;
-                    fs = q_mul(cs, IO::lds(st));
+                for (int o = 0; o < 8; o++) {
+                    // this thread's pieces of group o have landed when at most
+                    // NST - 1 younger copy groups are pending
+                    cp_async_wait<NST - 1>();
+                    Q4 fs = q_splat((TC)0);
+                    if (valid && active) {
+                        const TS *st = ring + (size_t)(o % NST) * (1 + DIM) * P + p0;
+                        fs = q_mul(cs, IO::lds(st));
 #pragma unroll
-                    for (int d = 0; d < DIM; d++) {
-                        const int L = list_of(o, d);
-                        const Q4 w = d < 2 ? q_splat(aw[L]) : (L == 4 ? dz0 : dz1);
-                        fs = q_fma(w, IO::lds(st + (1 + d) * P), fs);
-                    }
-                    if (xm & lists_of<DIM>(o)) {
-                        // further sources: the fine neighbours behind a coarse face
-#pragma unroll 1
                         for (int d = 0; d < DIM; d++) {
                             const int L = list_of(o, d);
-                            const Q4 da = d == 0 ? q_splat(dax) : (d == 1 ? q_splat(day) : daz);
-                            for (int k = 1; k < sl.cnt[L]; k++) {
-                                const int32_t src = sl.src[L * 4 + k];
-                                const Q4 v = IO::ldg(fin + (int64_t)(src & 0x0fffffff) * NV +
-                                                     (o ^ (src >> 28)) * P + p0);
-                                fs = q_fma(q_mul(da, q_splat(sl.w[L * 4 + k])), v, fs);
+                            const Q4 w = d < 2 ? q_splat(aw[L]) : (L == 4 ? dz0 : dz1);
+                            fs = q_fma(w, IO::lds(st + (1 + d) * P), fs);
+                        }
+                        if constexpr (decltype(more)::value) {
+                            // the fine neighbours behind a coarse face
+#pragma unroll 1
+                            for (uint32_t m = xm & entries_of<DIM>(o); m; m &= m - 1) {
+                                const int e = __ffs(m) - 1;
+                                const int32_t src = sl.src[e];
+                                const Q4 da = e < 8 ? q_splat(dax) : (e < 16 ? q_splat(day) : daz);
+                                const Q4 v = IO::ldg(fin_p0 + ((int64_t)(src & 0x0fffffff) * 8 + (o ^ (src >> 28))) * P);
+                                fs = q_fma(q_mul(da, q_splat(sl.w[e])), v, fs);
                             }
                         }
                     }
+                    cur[o] = fs;
+                    // refill the stage, NST groups ahead: groups 4..7 of this cell,
+                    // then groups 0..3 of the next one
+                    if (o == 8 - NST) on = point(j + 1);
+                    copy_group(on, (o + NST) & 7, o % NST, dep_of(fs));
                 }
-                cur[o] = fs;
-                if (active && nxt >= 0) prefetch_l2(pf + o * P);
-                // refill the stage, NST groups ahead: groups 4..7 of this cell,
-                // then groups 0..3 of the next one
-                if (o == NST) on = point(j + 1);
-                copy_group(on, (o + NST) & 7, o % NST, dep_of(fs));
+            };
+            // Cells without further sources take a copy of the loop without
+            // their branch, in which the loads of several groups are scheduled
+            // together (24^3, 159k cells: BF16 4.39 -> 4.02 ms, FP32 4.41 ->
+            // 4.38).  Three small CTAs an SM (16^3) hide the further sources'
+            // latency for one another, and one loop with those added at its
+            // end is the faster form (27k cells, four steps: 1.28 -> 1.18
+            // ms;
+            // at 24^3, where nothing else runs meanwhile, it takes 6.6 ms).
+            if constexpr (PC == 512) {
+                transport(std::false_type{});
+#pragma unroll 1
+                for (uint32_t m = valid && active ? xm : 0u; m; m &= m - 1) {
+                    const int e = __ffs(m) - 1, d = e >> 3;
+                    const int32_t src = sl.src[e];
+                    const Q4 w = q_mul(d == 0 ? q_splat(dax) : (d == 1 ? q_splat(day) : daz), q_splat(sl.w[e]));
+                    const TS *at = fin_p0 + (int64_t)(src & 0x0fffffff) * NV;
+                    // bit o: group o takes the entry's list
+                    const int groups = (d == 0 ? 0xf0 : (d == 1 ? 0xcc : 0xaa)) ^ ((e & 4) ? 0xff : 0);
+#pragma unroll
+                    for (int o = 0; o < 8; o++)
+                        if ((groups >> o) & 1) cur[o] = q_fma(w, IO::ldg(at + (o ^ (src >> 28)) * P), cur[o]);
+                }
+            } else if (xm) {
+                transport(std::true_type{});
+            } else {
+                transport(std::false_type{});
             }
         }
         if (valid) {
