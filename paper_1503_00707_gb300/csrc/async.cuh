@@ -124,9 +124,6 @@ __device__ inline void cp_async16_zfill(uint32_t dst, const void *src, uint32_t 
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-// Prefetch of the line holding src into L2.
-__device__ inline void prefetch_l2(const void *src) { asm volatile("prefetch.global.L2 [%0];" ::"l"(src)); }
-
 // Bulk prefetch of [src, src + bytes) into L2 (bytes a multiple of 16).
 __device__ inline void prefetch_l2_bulk(const void *src, uint32_t bytes)
 {

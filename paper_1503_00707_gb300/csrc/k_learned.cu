@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
     __shared__ float4 ZT[MAXN];  // (exp(-cz^2/2), d3 cz + d4 cz^2, cz^2/2, 0)
     __shared__ float os[64];
     __shared__ double sums[3][14];
+    __shared__ ffn psum[42][6];
     __shared__ double rred[2][5];
     __shared__ double cc[5];
     __shared__ double ered[AT / 32], qred[AT / 32];
@@ -320,7 +321,10 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
     const int nv = n.x * n.y * n.z;
     const uint32_t bytes = (uint32_t)nv * 4u;
     float *tile = dsm;                                             // [nv]
-    float4 *S2 = reinterpret_cast<float4 *>(dsm + nv);            // [ny][nz]: modes a = 0..3
+    // [ny][nz + 1]: modes a = 0..3 (a warp's lanes read one column of
+    // consecutive rows: 16-byte words nz + 1, odd, apart fall in different banks)
+    float4 *S2 = reinterpret_cast<float4 *>(dsm + nv);
+    const int lds2 = n.z + 1;
     if (tid == 0) {
         mbar_init(&bar, 1);
         abort_flag = 0;
@@ -357,11 +361,13 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
     // numbers split exactly by FMA; FP64 would run on this GPU's narrow FP64
     // pipe): the term these tables define then has its moments, and the
     // correction below closes them, to double-float rounding
-    if (tid < 42) {
-        const int d = tid / 14, k = tid % 14;
+    // (sum s on threads 6 s .. 6 s + 5, a sixth of the nodes each)
+    if (tid < 252) {
+        const int q = tid / 6, part = tid - 6 * q;
+        const int d = q / 14, k = q % 14;
         const int nd = d == 0 ? n.x : (d == 1 ? n.y : n.z);
         ffn s{0.0f, 0.0f};
-        for (int i = 0; i < nd; i++) {
+        for (int i = part; i < nd; i += 6) {
             const float4 h = H[d][i];
             const float c = G[d][i];
             int pw;
@@ -377,10 +383,10 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
             // t = e (or e He_a) times c^pw, as a double-float product
             const float p0 = k < 5 ? w0 : h.w * w0;
             ffn t{p0, k < 5 ? 0.0f : fmaf(h.w, w0, -p0)};
-            for (int q = 0; q < pw; q++) t = t * c;
+            for (int m = 0; m < pw; m++) t = t * c;
             s = s + t;
         }
-        sums[d][k] = (double)s.hi + (double)s.lo;
+        psum[q][part] = s;
     }
     // S1[4a+b][iz] = sum_c o_abc He_c(iz)
     for (int idx = tid; idx < 16 * nz; idx += AT) {
@@ -390,6 +396,12 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
         S1[ab][iz] = om[0] + om[1] * h.x + om[2] * h.y + om[3] * h.z;
     }
     __syncthreads();
+    if (tid < 42) {
+        ffn s = psum[tid][0];
+#pragma unroll
+        for (int m = 1; m < 6; m++) s = s + psum[tid][m];
+        sums[tid / 14][tid % 14] = (double)s.hi + (double)s.lo;
+    }
     // S2[iy][iz][a] = sum_b S1[4a+b][iz] He_b(iy)
     for (int idx = tid; idx < n.y * nz; idx += AT) {
         const int iy = idx / nz, iz = idx - iy * nz;
@@ -398,8 +410,9 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
 #pragma unroll
         for (int a = 0; a < 4; a++)
             r[a] = S1[4 * a][iz] + S1[4 * a + 1][iz] * h.x + S1[4 * a + 2][iz] * h.y + S1[4 * a + 3][iz] * h.z;
-        S2[idx] = make_float4(r[0], r[1], r[2], r[3]);
+        S2[iy * lds2 + iz] = make_float4(r[0], r[1], r[2], r[3]);
     }
+    __syncthreads();
     // moments of the reconstructed term: sum_m o_m R_r(m), R_r = sum e H_m phi_r
     if (tid < 64) {
         const int a = tid >> 4, b = (tid >> 2) & 3, c = tid & 3;
@@ -538,7 +551,7 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
         const float K0 = d0 + d1 * gx + d2 * gy + d4 * (gx * gx + gy * gy - 3.0f);
         const float Pxy = Mcf * hx.w * hy.w;
         const float Lxy = lnMc - 0.5f * (gx * gx + gy * gy);
-        const float4 *s2row = S2 + iy * nz;
+        const float4 *s2row = S2 + iy * lds2;
 #pragma unroll
         for (int sz = 0; sz < 2; sz++) {
             const int base = (4 * sx + 2 * sy + sz) * P + (mx * Hy + my) * Hz;
@@ -559,10 +572,13 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
             }
         }
     };
+    // one pass: the entropy sums, and f + dt/Kn Q into the tile, which is
+    // stored only if the checks hold
     float ent = 0.0f, qabs = 0.0f;
     if (good) {
         for (int pp = tid; pp < n.x * n.y; pp += AT)
-            pencil(pp, [&](float4 *, const float (&fv)[4], const float (&Q)[4], const float (&lnM)[4], int) {
+            pencil(pp, [&](float4 *fp, const float (&fv)[4], const float (&Q)[4], const float (&lnM)[4], int) {
+                float fn[4];
 #pragma unroll
                 for (int e = 0; e < 4; e++) {
                     const float x = fv[e];
@@ -570,7 +586,9 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
                     const float lf = x >= 1.17549435e-38f ? __logf(x) : (x > 0.0f ? logf(x) : -690.77552789821f);
                     ent = fmaf(Q[e], lf - lnM[e], ent);
                     qabs += fabsf(Q[e]);
+                    fn[e] = fmaf(dtkn, Q[e], x);
                 }
+                *fp = make_float4(fn[0], fn[1], fn[2], fn[3]);
             });
     }
     // warp sums in FP32 (their rounding is far below the gate's 1e-5), the
@@ -604,13 +622,13 @@ __global__ void __launch_bounds__(AT) k_lapply(float *__restrict__ f, const doub
         }
         return;
     }
-    float *qc = q_out ? q_out + cell * nv : nullptr;
-    for (int pp = tid; pp < n.x * n.y; pp += AT)
-        pencil(pp, [&](float4 *fp, const float (&fv)[4], const float (&Q)[4], const float (&)[4], int v) {
-            *fp = make_float4(fmaf(dtkn, Q[0], fv[0]), fmaf(dtkn, Q[1], fv[1]), fmaf(dtkn, Q[2], fv[2]),
-                              fmaf(dtkn, Q[3], fv[3]));
-            if (qc) *reinterpret_cast<float4 *>(qc + v) = make_float4(Q[0], Q[1], Q[2], Q[3]);
-        });
+    if (q_out) {
+        float *qc = q_out + cell * nv;
+        for (int pp = tid; pp < n.x * n.y; pp += AT)
+            pencil(pp, [&](float4 *, const float (&)[4], const float (&Q)[4], const float (&)[4], int v) {
+                *reinterpret_cast<float4 *>(qc + v) = make_float4(Q[0], Q[1], Q[2], Q[3]);
+            });
+    }
     fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
@@ -664,11 +682,13 @@ int launch_learned_apply(float *f, const double *mom, const float *o, const floa
 {
     if (!grid_ok(n)) return DVM_ENOTIMPL;
     if (ncells <= 0) return DVM_OK;
+    // 200 KB of tile and table, and the table's padding
     const size_t dyn = (size_t)n[0] * n[1] * n[2] * sizeof(float) + (size_t)n[1] * n[2] * sizeof(float4);
     if (dyn > 200 * 1024) return DVM_ENOTIMPL;
-    if (cudaFuncSetAttribute(k_lapply, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+    const size_t pad = (size_t)n[1] * sizeof(float4);
+    if (cudaFuncSetAttribute(k_lapply, cudaFuncAttributeMaxDynamicSharedMemorySize, 201 * 1024) != cudaSuccess)
         return DVM_ECUDA;
-    k_lapply<<<(unsigned)ncells, AT, dyn, s>>>(f, mom, o, o_eq, knl, thr, amag, make_int3(n[0], n[1], n[2]), (float)dtkn,
+    k_lapply<<<(unsigned)ncells, AT, dyn + pad, s>>>(f, mom, o, o_eq, knl, thr, amag, make_int3(n[0], n[1], n[2]), (float)dtkn,
                                                 used, list, count, q_out, dV, res, status);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
