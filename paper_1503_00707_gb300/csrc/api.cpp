@@ -1918,6 +1918,10 @@ int dvm_lbm_step(dvm_ctx *c, int nsteps, double dt, double tau)
     p.lev = c->d_llev;
     p.dt = dt;
     p.omega = dt / tau;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    p.threads = dvm::lbm_threads(p.ncells, nsm);
     p.status = c->d_lstatus;
     p.stream = c->stream;
     for (int s = 0; s < nsteps; s++) {
@@ -1942,15 +1946,11 @@ int dvm_lbm_moments(dvm_ctx *c, double *rho, double *u)
     const int64_t nc = ncells_of(c);
     int rc = dvm::launch_lbm_moments(c->cfg.precision, c->lat.q, c->d_lf[c->lcur], nc, c->lbm_ld, c->d_lmom, c->stream);
     if (rc) return fail(c, rc, "lattice Boltzmann moments launch");
-    std::vector<double> m((size_t)nc * 4);
-    rc = cuda_check(c, cudaMemcpyAsync(m.data(), c->d_lmom, m.size() * 8, cudaMemcpyDeviceToHost, c->stream), "moments");
-    if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "moments");
-    if (rc) return rc;
-    for (int64_t q = 0; q < nc; q++) {
-        rho[q] = m[4 * q];
-        for (int d = 0; d < 3; d++) u[3 * q + d] = m[4 * q + 1 + d];
-    }
-    return DVM_OK;
+    // rho and u lie on the device as the caller takes them
+    rc = cuda_check(c, cudaMemcpyAsync(rho, c->d_lmom, (size_t)nc * 8, cudaMemcpyDeviceToHost, c->stream), "moments");
+    if (!rc) rc = cuda_check(c, cudaMemcpyAsync(u, c->d_lmom + nc, (size_t)nc * 24, cudaMemcpyDeviceToHost, c->stream), "moments");
+    const int rs = cuda_check(c, cudaStreamSynchronize(c->stream), "moments");
+    return rc ? rc : rs;
 }
 
 int dvm_launch_count(int64_t *count)

@@ -117,17 +117,21 @@ template <int NS> struct ForS<NS, NS> {
 };
 
 // g_i += w f_e for every velocity i that takes side K, f_e the source's
-// value of velocity i (or of its mirror along the side's axis for a wall)
-template <typename T, int Q, int K>
-__device__ __forceinline__ void add_side(T (&g)[Q], const T *__restrict__ fin, int64_t ld, int64_t src, bool wall,
-                                         T w)
+// value of velocity i (or of its mirror along the side's axis for a wall;
+// WALLS: the side may be one)
+template <typename T, int Q, int K, bool WALLS>
+__device__ __forceinline__ void add_side(T (&g)[Q], const T *__restrict__ fin, int64_t ld, uint32_t src, bool wall, T w)
 {
     constexpr int d = K / 2;
     ForV<0, Q>::run([&](auto II) {
         constexpr int i = decltype(II)::value;
         if constexpr (Lat<Q>::t.c[i][d] != 0 && side_of<Q>(i, d) == K) {
-            constexpr int jm = Lat<Q>::t.mirror[i][d];
-            g[i] += w * __ldg(fin + (int64_t)(wall ? jm : i) * ld + src);
+            if constexpr (WALLS) {
+                constexpr int jm = Lat<Q>::t.mirror[i][d];
+                g[i] += w * __ldg(fin + (int64_t)(wall ? jm : i) * ld + src);
+            } else {
+                g[i] += w * __ldg(fin + (int64_t)i * ld + src);
+            }
         }
     });
 }
@@ -149,6 +153,7 @@ template <typename T, int DIM, int Q>
 __global__ void __launch_bounds__(256, lbm_min_blocks(Q, sizeof(T))) k_lbm(const LbmParams p)
 {
     const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned lanes = __ballot_sync(0xffffffffu, cell < p.ncells);
     if (cell >= p.ncells) return;
     const T *__restrict__ fin = static_cast<const T *>(p.f_in);
     T *__restrict__ fout = static_cast<T *>(p.f_out);
@@ -170,31 +175,46 @@ __global__ void __launch_bounds__(256, lbm_min_blocks(Q, sizeof(T))) k_lbm(const
         g[i] = v - dth * T(na) * v;
     });
     // transport, Eq. 2: add dt m_e f_e / (2^(dim-1) h) over each upwind
-    // side's sources, first sources for all sides at once
-    bool any_ovf = false;
-    ForS<0, NS>::run([&](auto KK) {
-        constexpr int k = decltype(KK)::value;
-        uint32_t e = code[k];
-        if (e & LBM_OVF) {
-            any_ovf = true;
-            e = __ldg(p.ovf + (e & LBM_CELL));
-        }
-        add_side<T, Q, k>(g, fin, ld, e & LBM_CELL, (e & LBM_WALL) != 0,
-                          dtq * T((int)((e >> LBM_M_SHIFT) & 3u) + 1));
-    });
-    if (any_ovf) {
+    // side's sources, first sources for all sides at once.  Warps without a
+    // wall or a side with several sources, most of them, take the copy without
+    // the choice of a mirrored row per gather (602k cells D3Q19 FP32, 0.19 GB
+    // a step and its codes: 31.9 -> 25.0 us; the kernel waits on its gathers
+    // and issues 59% of the cycles; 3, 5 and 6 CTAs an SM 28.4, 30.1, 32.8 us).
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < NS; k++) any |= code[k];
+    if (!__any_sync(lanes, any & (LBM_OVF | LBM_WALL))) {
         ForS<0, NS>::run([&](auto KK) {
             constexpr int k = decltype(KK)::value;
-            if (code[k] & LBM_OVF) {
-                const uint32_t base = code[k] & LBM_CELL;
-                const int n = (int)((code[k] >> LBM_M_SHIFT) & 3u) + 1;
-                for (int j = 1; j < n; j++) {
-                    const uint32_t e = __ldg(p.ovf + base + j);
-                    add_side<T, Q, k>(g, fin, ld, e & LBM_CELL, (e & LBM_WALL) != 0,
-                                      dtq * T((int)((e >> LBM_M_SHIFT) & 3u) + 1));
-                }
-            }
+            add_side<T, Q, k, false>(g, fin, ld, code[k] & LBM_CELL, false,
+                                     dtq * T((int)((code[k] >> LBM_M_SHIFT) & 3u) + 1));
         });
+    } else {
+        bool any_ovf = false;
+        ForS<0, NS>::run([&](auto KK) {
+            constexpr int k = decltype(KK)::value;
+            uint32_t e = code[k];
+            if (e & LBM_OVF) {
+                any_ovf = true;
+                e = __ldg(p.ovf + (e & LBM_CELL));
+            }
+            add_side<T, Q, k, true>(g, fin, ld, e & LBM_CELL, (e & LBM_WALL) != 0,
+                                    dtq * T((int)((e >> LBM_M_SHIFT) & 3u) + 1));
+        });
+        if (any_ovf) {
+            ForS<0, NS>::run([&](auto KK) {
+                constexpr int k = decltype(KK)::value;
+                if (code[k] & LBM_OVF) {
+                    const uint32_t base = code[k] & LBM_CELL;
+                    const int n = (int)((code[k] >> LBM_M_SHIFT) & 3u) + 1;
+                    for (int j = 1; j < n; j++) {
+                        const uint32_t e = __ldg(p.ovf + base + j);
+                        add_side<T, Q, k, true>(g, fin, ld, e & LBM_CELL, (e & LBM_WALL) != 0,
+                                                dtq * T((int)((e >> LBM_M_SHIFT) & 3u) + 1));
+                    }
+                }
+            });
+        }
     }
     // moments of f*
     T rho = T(0), jx = T(0), jy = T(0), jz = T(0);
@@ -225,30 +245,75 @@ __global__ void __launch_bounds__(256, lbm_min_blocks(Q, sizeof(T))) k_lbm(const
     });
 }
 
+// rho [ncells] and u [ncells][3] of the stored f in FP64.  FP32 values are
+// summed exactly on the FP32 pipe (FP64 runs at 1/64 of its rate): each splits
+// without error against 2^k > 32 max|f| into a multiple of 2^(k-24), a multiple
+// of 2^(k-42) and a rest, and the sums of either multiple over a cell are exact
+// in FP32 (the extraction of Rump, Ogita and Oishi, 2008).  602k cells
+// D3Q19: the FP64 sums took 136 us.
 template <typename T, int Q>
 __global__ void __launch_bounds__(256) k_lbm_moments(const T *__restrict__ f, int64_t ncells, int64_t ld,
                                                      double *__restrict__ out)
 {
     const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (cell >= ncells) return;
-    double rho = 0, j[3] = {0, 0, 0};
+    T v[Q];
     ForV<0, Q>::run([&](auto II) {
         constexpr int i = decltype(II)::value;
-        constexpr int cx = Lat<Q>::t.c[i][0], cy = Lat<Q>::t.c[i][1], cz = Lat<Q>::t.c[i][2];
-        const double v = (double)f[(int64_t)i * ld + cell];
-        rho += v;
-        j[0] += cx * v;
-        j[1] += cy * v;
-        j[2] += cz * v;
+        v[i] = __ldg(f + (int64_t)i * ld + cell);
     });
-    out[cell * 4] = rho;
-    for (int d = 0; d < 3; d++) out[cell * 4 + 1 + d] = j[d] / rho;
+    // s[0] = sum x_i, s[1 + d] = sum c_id x_i
+    auto sums = [&](const T(&x)[Q], auto &s) {
+        ForV<0, Q>::run([&](auto II) {
+            constexpr int i = decltype(II)::value;
+            constexpr int cx = Lat<Q>::t.c[i][0], cy = Lat<Q>::t.c[i][1], cz = Lat<Q>::t.c[i][2];
+            s[0] += x[i];
+            if constexpr (cx > 0) s[1] += x[i];
+            if constexpr (cx < 0) s[1] -= x[i];
+            if constexpr (cy > 0) s[2] += x[i];
+            if constexpr (cy < 0) s[2] -= x[i];
+            if constexpr (cz > 0) s[3] += x[i];
+            if constexpr (cz < 0) s[3] -= x[i];
+        });
+    };
+    double m[4] = {0, 0, 0, 0};
+    bool wide = true;
+    if constexpr (sizeof(T) == 4) {
+        uint32_t mx = 0;
+#pragma unroll
+        for (int i = 0; i < Q; i++) mx = max(mx, __float_as_uint(v[i]) & 0x7fffffffu);
+        const int ex = (int)(mx >> 23);  // max|f| < 2^(ex - 126)
+        wide = ex < 48 || ex > 240;
+        if (!wide) {
+            const float sg1 = __int_as_float((ex + 7) << 23), sg2 = __int_as_float((ex - 11) << 23);
+            float q[Q], s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0}, s3[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int i = 0; i < Q; i++) {
+                q[i] = __fadd_rn(__fadd_rn(v[i], sg1), -sg1);
+                v[i] -= q[i];
+            }
+            sums(q, s1);
+#pragma unroll
+            for (int i = 0; i < Q; i++) {
+                q[i] = __fadd_rn(__fadd_rn(v[i], sg2), -sg2);
+                v[i] -= q[i];
+            }
+            sums(q, s2);
+            sums(v, s3);
+#pragma unroll
+            for (int k = 0; k < 4; k++) m[k] = (double)s1[k] + ((double)s2[k] + (double)s3[k]);
+        }
+    }
+    if (wide) sums(v, m);
+    out[cell] = m[0];
+#pragma unroll
+    for (int d = 0; d < 3; d++) out[ncells + 3 * cell + d] = m[1 + d] / m[0];
 }
 
 template <typename T, int DIM, int Q> int launch_t(const LbmParams &p)
 {
-    const int64_t blocks = (p.ncells + 255) / 256;
-    k_lbm<T, DIM, Q><<<(unsigned)blocks, 256, 0, p.stream>>>(p);
+    const int t = p.threads;
+    k_lbm<T, DIM, Q><<<(unsigned)((p.ncells + t - 1) / t), t, 0, p.stream>>>(p);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
 }
@@ -275,6 +340,16 @@ int launch_mom_t(int q, const void *f, int64_t ncells, int64_t ld, double *out, 
 }
 
 }  // namespace
+
+// Threads per CTA: 256, fewer where that leaves SMs without a CTA (1,388
+// cells D2Q9 FP64 ran on six SMs, each bound by its FP64 pipe:
+// 14.5 -> 8.4 us a step).
+int lbm_threads(int64_t ncells, int nsm)
+{
+    int t = 256;
+    while (t > 32 && (ncells + t - 1) / t < nsm) t /= 2;
+    return t;
+}
 
 int launch_lbm(const LbmParams &p)
 {

@@ -52,12 +52,15 @@ struct LbmParams {
     const uint8_t *lev;       // [ncells]
     double dt, omega;         // omega = dt / tau
     int *status;              // bit 0: a cell with rho <= 0 or non-finite moments
+    int threads;              // per CTA, from lbm_threads
     cudaStream_t stream;
 };
 
+int lbm_threads(int64_t ncells, int nsm);
+
 int launch_lbm(const LbmParams &p);
 
-// rho, u of every cell in FP64: out [ncells][4]
+// rho, u of every cell in FP64: out rho [ncells], then u [ncells][3]
 int launch_lbm_moments(int prec, int q, const void *f, int64_t ncells, int64_t ld, double *out,
                        cudaStream_t s);
 
