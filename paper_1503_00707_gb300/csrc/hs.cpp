@@ -441,7 +441,7 @@ void pack_warp(const std::vector<int> &nodes, std::vector<std::vector<PackTrial>
     long total = 0;
     for (int k = 0; k < kn; k++) total += (long)tr[k].size();
     uint64_t st = mix64(seed);
-    for (long it = 0; it < (kind ? 60 : 30) * total && R > 1; it++) {
+    for (long it = 0; it < (kind ? 200 : 100) * total && R > 1; it++) {
         st = mix64(st);
         const int k = (int)(st % (uint64_t)kn);
         const int e1 = (int)((st >> 16) % (uint64_t)R), e2 = (int)((st >> 32) % (uint64_t)R);
@@ -449,7 +449,7 @@ void pack_warp(const std::vector<int> &nodes, std::vector<std::vector<PackTrial>
         int &p1 = at[(size_t)l1 * HM + e1], &p2 = at[(size_t)l2 * HM + e2];
         HalfSlot &h1 = half(l1, e1), &h2 = half(l2, e2);
         if (&h1 == &h2 || (p1 < 0 && p2 < 0)) continue;
-        if ((p1 < 0 && h2.wave == ng) || (p2 < 0 && h1.wave == ng)) continue;  // nothing to gain by a move
+        if (h1.wave == ng && h2.wave == ng) continue;  // neither slot has a conflict
         // the trials before, and after the exchange (l and m flipped at will)
         PackTrial o1{}, o2{}, n1{}, n2{};
         if (p1 >= 0) n1 = o1 = tr[k][p1];
