@@ -62,6 +62,8 @@ struct dvm_ctx {
     int64_t tsteps = 0;
     int *d_status = nullptr;
     unsigned long long *d_counter = nullptr;
+    unsigned int *d_done = nullptr;
+    dvm::StepPlan plan;  // of the current velocity grid
     bool have_step_moments = false;
     bool mesh_on_device = false;
     dvm::HsTables hs;
@@ -213,6 +215,7 @@ int ensure_device(dvm_ctx *c)
     }
     // the step kernel's cell dispenser shares the allocation
     c->d_counter = reinterpret_cast<unsigned long long *>(c->d_status + 2);
+    c->d_done = reinterpret_cast<unsigned int *>(c->d_status + 1);
     return DVM_OK;
 }
 
@@ -719,6 +722,7 @@ int dvm_set_velocity_grid(dvm_ctx *c, const int n[3], const double lo[3], const 
         c->hi[d] = hi[d];
         c->hv[d] = (hi[d] - lo[d]) / n[d];
     }
+    c->plan = dvm::StepPlan{};
     c->dV = c->hv[0] * c->hv[1] * c->hv[2];
     c->nv = n[0] * n[1] * n[2];
     c->P = c->nv / 8;
@@ -1006,6 +1010,8 @@ int dvm_step(dvm_ctx *c, int nsteps, double dt)
     p.mom_out = c->d_mom;
     p.status = c->d_status;
     p.counter = c->d_counter;
+    p.done = c->d_done;
+    p.plan = &c->plan;
     p.stream = c->stream;
     // the BGK step kernel writes the residual of its collision term; the
     // hard-sphere and learned updates write theirs after the transport launch
@@ -1025,10 +1031,6 @@ int dvm_step(dvm_ctx *c, int nsteps, double dt)
         p.res_out = nullptr;
         p.res_phi = bgk ? reinterpret_cast<float2 *>(c->d_res) : nullptr;
         if (c->timing) cudaEventRecord(c->tev[0], c->stream);
-        if (cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(c, DVM_ECUDA, "counter reset failed");
-        }
         int rc = dvm::launch_step(p);
         if (rc) return fail(c, rc, rc == DVM_ENOTIMPL ? "velocity grid too large for the step kernel" : "step launch failed");
         if (c->timing) cudaEventRecord(c->tev[1], c->stream);
@@ -1230,6 +1232,7 @@ int dvm_step_partitioned(dvm_ctx *c, int nparts, int nsteps, double dt)
     base.dV = c->dV;
     base.status = c->d_status;
     base.counter = c->d_counter;
+    base.done = c->d_done;
     base.stream = c->stream;
     for (int s = 0; s < nsteps && !rc; s++) {
         const int b = s & 1;
@@ -1247,8 +1250,7 @@ int dvm_step_partitioned(dvm_ctx *c, int nparts, int nsteps, double dt)
             q.st_cnt = c->d_cnt + pt.c0 * 8;
             q.inv_h = static_cast<const char *>(c->d_invh) + pt.c0 * tcs;
             q.mom_out = dev[p].mom;
-            rc = cuda_check(c, cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream), "counter reset");
-            if (!rc) rc = dvm::launch_step(q);
+            rc = dvm::launch_step(q);
             if (rc && rc != DVM_ECUDA) rc = fail(c, rc, "step launch failed");
         }
     }
@@ -1527,12 +1529,11 @@ int dvm_mlp_forward(dvm_ctx *c, const float *x, int64_t n, float *y)
     if (!c->mlp_set) return fail(c, DVM_ESTATE, "no weights set");
     int rc = dvm::mlp_reserve(c->mlp, n, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
     if (rc) return fail(c, rc, "device allocation (network work buffers)");
-    DevArr dx(c, (size_t)n * 64 * 4), dy(c, (size_t)n * 64 * 4);
-    if (!dx.p || !dy.p) return fail(c, DVM_ENOMEM, "device allocation (network rows)");
-    rc = cuda_check(c, cudaMemcpyAsync(dx.p, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
-    if (!rc) rc = dvm::mlp_forward(c->mlp, dx.f(), n, dy.f(), c->d_status, c->stream);
+    float *dx = c->mlp.rows(0), *dy = c->mlp.rows(1);
+    rc = cuda_check(c, cudaMemcpyAsync(dx, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
+    if (!rc) rc = dvm::mlp_forward(c->mlp, dx, n, dy, c->d_status, c->stream);
     if (rc) return fail(c, rc, "network forward failed");
-    rc = cuda_check(c, cudaMemcpyAsync(y, dy.p, (size_t)n * 256, cudaMemcpyDeviceToHost, c->stream), "copy y");
+    rc = cuda_check(c, cudaMemcpyAsync(y, dy, (size_t)n * 256, cudaMemcpyDeviceToHost, c->stream), "copy y");
     return rc ? rc : status_check(c);
 }
 
@@ -1542,11 +1543,10 @@ int dvm_mlp_loss_grad(dvm_ctx *c, const float *x, const float *t, int64_t n, flo
     if (!c->mlp_set) return fail(c, DVM_ESTATE, "no weights set");
     int rc = dvm::mlp_reserve(c->mlp, n, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
     if (rc) return fail(c, rc, "device allocation (network work buffers)");
-    DevArr dx(c, (size_t)n * 256), dt(c, (size_t)n * 256);
-    if (!dx.p || !dt.p) return fail(c, DVM_ENOMEM, "device allocation (network rows)");
-    rc = cuda_check(c, cudaMemcpyAsync(dx.p, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
-    if (!rc) rc = cuda_check(c, cudaMemcpyAsync(dt.p, t, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy t");
-    if (!rc) rc = dvm::mlp_grad(c->mlp, dx.f(), dt.f(), n, c->d_status, c->stream);
+    float *dx = c->mlp.rows(0), *dt = c->mlp.rows(1);
+    rc = cuda_check(c, cudaMemcpyAsync(dx, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
+    if (!rc) rc = cuda_check(c, cudaMemcpyAsync(dt, t, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy t");
+    if (!rc) rc = dvm::mlp_grad(c->mlp, dx, dt, n, c->d_status, c->stream);
     if (rc) return fail(c, rc, "network gradient failed");
     double L = 0.0;
     rc = cuda_check(c, cudaMemcpyAsync(&L, c->mlp.loss, 8, cudaMemcpyDeviceToHost, c->stream), "copy loss");

@@ -480,7 +480,8 @@ int mlp_reserve(Mlp &m, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree
                          (size_t)np * 64 * 2, (size_t)np * 64 * 2,           // dO, dOt
                          (size_t)np * 256 * 2 * 2, (size_t)np * 256 * 2 * 3, // dZ (two in turn), dZt of each layer
                          (size_t)21 * MLP_NPARAM * 4,                        // partial weight gradients (at most 21 splits)
-                         tiles * 832 * 4, tiles * 8};                        // partial bias gradients and losses
+                         tiles * 832 * 4, tiles * 8,                         // partial bias gradients and losses
+                         (size_t)np * 256, (size_t)np * 256};                // a host call's rows
     static_assert(sizeof(sz) / sizeof(sz[0]) == MLP_NWORK, "work buffer count");
     for (int i = 0; i < MLP_NWORK; i++) {
         m.work[i].p = alloc(sz[i]);

@@ -820,6 +820,15 @@ __global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_s
             }
             bar_arrive_n(BAR_C + q, nbar);
         }
+        // the last solver warp to get here leaves the dispenser as it was (a
+        // memset before each launch cost a short step its launch and gap)
+        if (lane == 0) {
+            __threadfence();
+            if (atomicAdd(p.done, 1u) == 2u * gridDim.x - 1u) {
+                *p.counter = 0ull;
+                *p.done = 0u;
+            }
+        }
         return;
     }
 
@@ -1087,18 +1096,27 @@ int launch_kernel(const StepParams &p, int ncw)
     auto kern = k_step<TS, DIM, COLL, PC>;
     const int threads = (ncw + 2) * 32;
     const size_t dyn = step_dyn_bytes<TS, DIM>(p.P);
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return DVM_ECUDA;
-    int dev = 0, optin = 0, nsm = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (fa.sharedSizeBytes + dyn > (size_t)optin) return DVM_ENOTIMPL;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-        return DVM_ECUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, dyn) != cudaSuccess || occ < 1)
-        return DVM_ENOTIMPL;
-    const int64_t grid = std::min<int64_t>(p.ncells, (int64_t)nsm * occ);
+    // the queries below take longer than a small step's launch: made once per
+    // plan.  The shared-memory limit is set to the device's own, so that
+    // contexts of different grids agree on it.
+    int64_t slots = p.plan ? p.plan->slots : 0;
+    if (!slots) {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return DVM_ECUDA;
+        int dev = 0, optin = 0, nsm = 0, occ = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (fa.sharedSizeBytes + dyn > (size_t)optin) return DVM_ENOTIMPL;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) !=
+            cudaSuccess)
+            return DVM_ECUDA;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, dyn) != cudaSuccess || occ < 1)
+            return DVM_ENOTIMPL;
+        slots = (int64_t)nsm * occ;
+        if (p.plan) p.plan->slots = slots;
+    }
+    const int64_t grid = std::min<int64_t>(p.ncells, slots);
     kern<<<(unsigned)grid, threads, dyn, p.stream>>>(p);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;

@@ -38,8 +38,15 @@ struct StepParams {
     float2 *res_phi;         // [ncells][5] or null: sum_i phi_r (M~ - f*)_i dV of the BGK
                              // step, phi = (1, c, |c|^2 - 3), as double-float pairs
     int *status;
-    unsigned long long *counter;  // cell dispenser of the step kernel, zeroed before each launch
+    unsigned long long *counter;  // cell dispenser of the step kernel and the count of its solver
+    unsigned int *done;           // warps that are through: zero before and after each launch
+    struct StepPlan *plan;        // launch shape kept by the caller for its grid and precision, or null
     cudaStream_t stream;
+};
+
+// Launch shape of the step kernel: resident CTAs on the device (0: not yet known).
+struct StepPlan {
+    int64_t slots = 0;
 };
 
 int launch_step(const StepParams &p);

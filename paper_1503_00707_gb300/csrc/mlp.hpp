@@ -12,7 +12,7 @@ namespace dvm {
 // W2[256][256] b2 W3[256][256] b3 W4[64][256] b4[64] (W[out][in]).
 constexpr int64_t MLP_NPARAM = 164672;
 
-enum { W_X = 0, W_XT, W_Z, W_H, W_HT, W_DO, W_DOT, W_DZ, W_DZT, W_PART, W_BIAS, W_LOSS, MLP_NWORK };
+enum { W_X = 0, W_XT, W_Z, W_H, W_HT, W_DO, W_DOT, W_DZ, W_DZT, W_PART, W_BIAS, W_LOSS, W_R0, W_R1, MLP_NWORK };
 
 struct DevBuf {
     void *p = nullptr;
@@ -34,6 +34,8 @@ struct Mlp {
     int64_t steps = 0;
     int64_t cap = 0;  // rows the work buffers hold (multiple of 64)
     DevBuf work[MLP_NWORK];
+    // rows [cap][64] of a host call's inputs, targets or outputs
+    float *rows(int k) { return static_cast<float *>(work[W_R0 + k].p); }
 };
 
 using DevAllocF = std::function<void *(size_t)>;

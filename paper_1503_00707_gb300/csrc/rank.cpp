@@ -48,6 +48,8 @@ struct dvm_rank {
     float *d_amag_f = nullptr;
     int *d_status = nullptr;
     unsigned long long *d_counter = nullptr;
+    unsigned int *d_done = nullptr;
+    dvm::StepPlan plan;
     std::vector<int64_t *> d_send, d_recv;    // per peer: local rows
     std::vector<int64_t> send_off, recv_off;
     int64_t *d_rows = nullptr;                // all peers' local rows
@@ -93,6 +95,7 @@ void free_device(dvm_rank *r)
     r->d_amag_f = nullptr;
     r->d_status = nullptr;
     r->d_counter = nullptr;
+    r->d_done = nullptr;
     r->d_rows = nullptr;
     r->d_send.clear();
     r->d_recv.clear();
@@ -267,6 +270,8 @@ int dvm_rank_set_velocity_grid(dvm_rank *r, const int n[3], const double lo[3], 
         return rfail(r, DVM_ENOMEM, "device allocation (rank)");
     }
     r->d_counter = reinterpret_cast<unsigned long long *>(r->d_status + 2);
+    r->d_done = reinterpret_cast<unsigned int *>(r->d_status + 1);
+    r->plan = dvm::StepPlan{};
     rc = check(r, cudaMemset(r->d_status, 0, 16), "status");
     // owned stencils: local sources, weights, counts and 1/h of cells c0 ..
     std::vector<double> invh(r->nown), w64((size_t)r->nown * 24);
@@ -433,9 +438,10 @@ int dvm_rank_step(dvm_rank *r, double dt)
     p.mom_out = r->d_mom;
     p.status = r->d_status;
     p.counter = r->d_counter;
+    p.done = r->d_done;
+    p.plan = &r->plan;
     p.stream = r->stream;
-    int rc = check(r, cudaMemsetAsync(r->d_counter, 0, sizeof(unsigned long long), r->stream), "counter reset");
-    if (!rc) rc = dvm::launch_step(p);
+    int rc = dvm::launch_step(p);
     if (rc) return rc == DVM_ECUDA ? rc : rfail(r, rc, "step launch failed");
     r->cur = 1 - r->cur;
     return read_status(r);
