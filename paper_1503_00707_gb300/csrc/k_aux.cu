@@ -4,6 +4,7 @@
 #include <cmath>
 
 #include "../../include/dvm.h"
+#include "async.cuh"
 #include "common.cuh"
 #include "kernels.hpp"
 #include "quads.cuh"
@@ -62,13 +63,20 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
 // weights that k_step's partials use (total size below 16 against the split's
 // margin), are exact in FP32 and go into 64-bit integers; the rests are summed
 // in FP32.  What is lost is below 2^-60 of sum |f|, less than FP64 summation
-// loses.  f is read once from HBM: a thread keeps its first two quads of
-// positions (32 values each) in registers between the search for M and the
-// sums; positions beyond that (grids of more than 512 quads) are read again.
-// A cell with non-finite values or M outside [2^-86, 2^115] takes FP64 sums.
-// 17,680 cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 319 us now
-// (3.1 TB/s, the registers of two quads a thread hold two CTAs an SM).
-constexpr int MOM_T = 256, MOM_HOLD = 2;
+// loses.  A cell with non-finite values or M outside [2^-86, 2^115] takes FP64
+// sums.
+//
+// f is read once from HBM and twice by its thread, for M and for the sums.
+// Cells of up to 56 KB go through shared memory (PIPE): a CTA takes every
+// gridDim-th cell, and each thread copies its own pieces of the next one with
+// cp.async while it sums this one, so that the stream does not stop for the
+// barriers and the FP64 tail of a cell.  Larger cells are read from memory
+// twice.  17,680 cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 319 us
+// with the cell held in registers (one cell per CTA), 283 us through
+// shared memory; what bounds it now is the arithmetic of the split at 14 warps
+// an SM.
+constexpr int MOM_T = 256;
+constexpr size_t MOM_ROW = 56 * 1024;
 
 __device__ inline uint32_t abs_bits(float2 v) { return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu); }
 
@@ -173,23 +181,33 @@ template <typename TC> __device__ inline void add_quad_f64(const QV<TC> (&x)[8],
     weighted_sums<double, double>(s, (double)jx, (double)jy, (double)jz, m);
 }
 
-template <typename TS>
+template <typename TS, bool PIPE>
 __global__ void __launch_bounds__(MOM_T, 2)
-    k_moments(const TS *__restrict__ f, int P, int3 half, double3 hh, double dV, double *__restrict__ out)
+    k_moments(const TS *__restrict__ f, int64_t ncells, int P, int3 half, double3 hh, double dV, double *__restrict__ out)
 {
     using IO = QIO<TS>;
     using TC = typename Store<TS>::TC;
     constexpr int VEC = Store<TS>::VEC;
+    extern __shared__ __align__(16) unsigned char mom_tile[];  // PIPE: [2][8 P]
     __shared__ uint32_t wmax[MOM_T / 32];
     __shared__ double red[MOM_T / 32][7];
     __shared__ int64_t redI[MOM_T / 32][7];
     __shared__ float redR[MOM_T / 32][7];
-    const int64_t c = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, nw = T >> 5, Q = P / VEC;
-    const TS *fc = f + c * 8 * (int64_t)P;
-    auto load = [&](int q, QV<TC> (&x)[8]) {
+    TS *tile = reinterpret_cast<TS *>(mom_tile);
+    // the thread's pieces of cell c into buffer b (each thread reads back only
+    // what it copied)
+    auto copy = [&](int64_t c, int b) {
+        if (c < ncells)
+            for (int q = tid; q < Q; q += T)
 #pragma unroll
-        for (int o = 0; o < 8; o++) x[o] = IO::ldg(fc + (int64_t)o * P + q * VEC);
+                for (int o = 0; o < 8; o++) {
+                    const TS *src = f + (c * 8 + o) * (int64_t)P + q * VEC;
+                    TS *dst = tile + (size_t)(b * 8 + o) * P + q * VEC;
+                    if constexpr (sizeof(TS) == 2) cp_async8(dst, src, 0u);
+                    else cp_async16(dst, src, 0u);
+                }
+        cp_async_commit();
     };
     auto nodes = [&](int q, int &jx, int &jy, int &jz) {
         const int p = q * VEC, t = p / half.z;
@@ -197,101 +215,105 @@ __global__ void __launch_bounds__(MOM_T, 2)
         jy = 2 * (t % half.y) + 1;
         jx = 2 * (t / half.y) + 1;
     };
-    int jx, jy, jz;
-    bool wide = true;  // FP64 sums
-    int ex = 0;
-    if constexpr (sizeof(TC) == 4) {
-        QV<float> x[MOM_HOLD][8];
-        uint32_t mx = 0;
-        auto top = [&](const QV<float> (&v)[8]) {
+    if constexpr (PIPE) copy(blockIdx.x, 0);
+    int buf = 0;
+    for (int64_t c = blockIdx.x; c < ncells; c += gridDim.x, buf ^= 1) {
+        if constexpr (PIPE) {
+            // the other buffer's values were all used before this cell's
+            // predecessor reached its barriers
+            copy(c + gridDim.x, buf ^ 1);
+            cp_async_wait<1>();
+        }
+        auto load = [&](int q, QV<TC> (&x)[8]) {
 #pragma unroll
-            for (int o = 0; o < 8; o++) mx = max(mx, max(abs_bits(v[o].a), abs_bits(v[o].b)));
+            for (int o = 0; o < 8; o++) {
+                if constexpr (PIPE) x[o] = IO::lds(tile + (size_t)(buf * 8 + o) * P + q * VEC);
+                else x[o] = IO::ldg(f + (c * 8 + o) * (int64_t)P + q * VEC);
+            }
         };
+        int jx, jy, jz;
+        bool wide = true;  // FP64 sums
+        int ex = 0;
+        if constexpr (sizeof(TC) == 4) {
+            uint32_t mx = 0;
+            for (int q = tid; q < Q; q += T) {
+                QV<float> x[8];
+                load(q, x);
 #pragma unroll
-        for (int h = 0; h < MOM_HOLD; h++)
-            if (tid + h * T < Q) load(tid + h * T, x[h]);
-#pragma unroll
-        for (int h = 0; h < MOM_HOLD; h++)
-            if (tid + h * T < Q) top(x[h]);
-        for (int q = tid + MOM_HOLD * T; q < Q; q += T) {
-            QV<float> y[8];
-            load(q, y);
-            top(y);
-        }
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (lane == 0) wmax[warp] = mx;
-        __syncthreads();
-        for (int w = 0; w < nw; w++) mx = max(mx, wmax[w]);
-        ex = (int)(mx >> 23);  // M < 2^(ex - 126)
-        wide = ex < 40 || ex > 240;
-        if (!wide) {
-            MomSum m{};
-#pragma unroll
-            for (int h = 0; h < MOM_HOLD; h++)
-                if (tid + h * T < Q) {
-                    nodes(tid + h * T, jx, jy, jz);
-                    add_quad(x[h], ex, jx, jy, jz, m);
+                for (int o = 0; o < 8; o++) mx = max(mx, max(abs_bits(x[o].a), abs_bits(x[o].b)));
+            }
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            if (lane == 0) wmax[warp] = mx;
+            __syncthreads();
+            for (int w = 0; w < nw; w++) mx = max(mx, wmax[w]);
+            ex = (int)(mx >> 23);  // M < 2^(ex - 126)
+            wide = ex < 40 || ex > 240;
+            if (!wide) {
+                MomSum m{};
+#pragma unroll 1
+                for (int q = tid; q < Q; q += T) {
+                    QV<float> x[8];
+                    load(q, x);
+                    nodes(q, jx, jy, jz);
+                    add_quad(x, ex, jx, jy, jz, m);
                 }
-#pragma unroll 1
-            for (int q = tid + MOM_HOLD * T; q < Q; q += T) {
-                QV<float> y[8];
-                load(q, y);
-                nodes(q, jx, jy, jz);
-                add_quad(y, ex, jx, jy, jz, m);
-            }
-            const int64_t I = warp_reduce7<int64_t>(m.I, lane);
-            const float R = warp_reduce7<float>(m.R, lane);
-            if ((lane & 3) == 0 && lane < 28) {
-                redI[warp][lane >> 2] = I;
-                redR[warp][lane >> 2] = R;
+                const int64_t I = warp_reduce7<int64_t>(m.I, lane);
+                const float R = warp_reduce7<float>(m.R, lane);
+                if ((lane & 3) == 0 && lane < 28) {
+                    redI[warp][lane >> 2] = I;
+                    redR[warp][lane >> 2] = R;
+                }
             }
         }
-    }
-    if (wide) {
-        double m[7] = {0, 0, 0, 0, 0, 0, 0};
-#pragma unroll 1
-        for (int q = tid; q < Q; q += T) {
-            QV<TC> y[8];
-            load(q, y);
-            nodes(q, jx, jy, jz);
-            add_quad_f64<TC>(y, jx, jy, jz, m);
-        }
-        const double t = warp_reduce7<double>(m, lane);
-        if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
-    }
-    __syncthreads();
-    if (warp) return;
-    double s = 0.0;
-    if (lane < 7) {
         if (wide) {
-            for (int w = 0; w < nw; w++) s += red[w][lane];
-        } else {
-            int64_t I = 0;
-            float R = 0.0f;
-            for (int w = 0; w < nw; w++) {
-                I += redI[w][lane];
-                R += redR[w][lane];
+            double m[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+            for (int q = tid; q < Q; q += T) {
+                QV<TC> x[8];
+                load(q, x);
+                nodes(q, jx, jy, jz);
+                add_quad_f64<TC>(x, jx, jy, jz, m);
             }
-            s = (double)I * __longlong_as_double((long long)(1023 + ex - 156) << 52) + (double)R;  // 2^(k-39)
+            const double t = warp_reduce7<double>(m, lane);
+            if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
         }
+        __syncthreads();
+        if (warp == 0) {
+            double s = 0.0;
+            if (lane < 7) {
+                if (wide) {
+                    for (int w = 0; w < nw; w++) s += red[w][lane];
+                } else {
+                    int64_t I = 0;
+                    float R = 0.0f;
+                    for (int w = 0; w < nw; w++) {
+                        I += redI[w][lane];
+                        R += redR[w][lane];
+                    }
+                    s = (double)I * __longlong_as_double((long long)(1023 + ex - 156) << 52) + (double)R;  // 2^(k-39)
+                }
+            }
+            // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
+            const double s0 = __shfl_sync(0xffffffffu, s, 0);
+            const int d = (lane + 2) % 3;
+            const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
+            const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
+            const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
+            const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
+                         uz2 = __shfl_sync(0xffffffffu, u2, 3);
+            const double ex2 = __shfl_sync(0xffffffffu, e2, 1), ey2 = __shfl_sync(0xffffffffu, e2, 2),
+                         ez2 = __shfl_sync(0xffffffffu, e2, 3);
+            double *o = out + c * 5;
+            if (lane == 0) {
+                o[0] = s0 * dV;
+                o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
+            } else if (lane < 4) {
+                o[lane] = v;
+            }
+        }
+        if (sizeof(TC) == 8) __syncthreads();  // red is read above (FP32: the next cell's first barrier)
     }
-    // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
-    const double s0 = __shfl_sync(0xffffffffu, s, 0);
-    const int d = (lane + 2) % 3;
-    const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
-    const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
-    const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
-    const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
-                 uz2 = __shfl_sync(0xffffffffu, u2, 3);
-    const double ex2 = __shfl_sync(0xffffffffu, e2, 1), ey2 = __shfl_sync(0xffffffffu, e2, 2),
-                 ez2 = __shfl_sync(0xffffffffu, e2, 3);
-    double *o = out + c * 5;
-    if (lane == 0) {
-        o[0] = s0 * dV;
-        o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
-    } else if (lane < 4) {
-        o[lane] = v;
-    }
+    if constexpr (PIPE) cp_async_wait_all();
 }
 
 template <typename TS>
@@ -320,6 +342,31 @@ int last_status()
 {
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
+}
+
+template <typename TS> int moments_t(const void *f, int64_t ncells, const MomGrid &g, double *out, cudaStream_t s)
+{
+    const int P = g.half[0] * g.half[1] * g.half[2], Q = P / Store<TS>::VEC;
+    // one quad a thread up to 256 quads, then two or more, evenly (24^3: 432
+    // quads on 224 threads)
+    const int rounds = (Q + MOM_T - 1) / MOM_T, t = ((Q + rounds - 1) / rounds + 31) / 32 * 32;
+    const int3 half = make_int3(g.half[0], g.half[1], g.half[2]);
+    const double3 hh = make_double3(0.5 * g.hv[0], 0.5 * g.hv[1], 0.5 * g.hv[2]);
+    const TS *ft = static_cast<const TS *>(f);
+    const size_t row = (size_t)8 * P * sizeof(TS);
+    if (row > MOM_ROW) {
+        k_moments<TS, false><<<(unsigned)ncells, t, 0, s>>>(ft, ncells, P, half, hh, g.dV, out);
+        return last_status();
+    }
+    auto kern = k_moments<TS, true>;
+    int dev = 0, nsm = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * MOM_ROW)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, t, 2 * row) != cudaSuccess || occ < 1)
+        return DVM_ECUDA;
+    kern<<<(unsigned)std::min<int64_t>(ncells, (int64_t)nsm * occ), t, 2 * row, s>>>(ft, ncells, P, half, hh, g.dV, out);
+    return last_status();
 }
 
 // Row copies between buffers: entry r of rows is {destination buffer, row,
@@ -430,21 +477,12 @@ int launch_init_maxwellian(int prec, void *f, int64_t ncells, int nv, int nmix, 
 int launch_moments(int prec, const void *f, int64_t ncells, const MomGrid &g, double *out, cudaStream_t s)
 {
     if (ncells <= 0) return DVM_OK;
-    const int P = g.half[0] * g.half[1] * g.half[2], Q = P / (prec == DVM_F64 ? 2 : 4);
-    // one quad a thread up to 256 quads, then two (24^3: 432 quads on 224 threads)
-    const int per = Q <= MOM_T ? Q : (Q + 1) / 2, t = std::min(MOM_T, (per + 31) / 32 * 32);
-    const dim3 grid((unsigned)ncells);
-    const int3 half = make_int3(g.half[0], g.half[1], g.half[2]);
-    const double3 hh = make_double3(0.5 * g.hv[0], 0.5 * g.hv[1], 0.5 * g.hv[2]);
     switch (prec) {
-    case DVM_F64: k_moments<double><<<grid, t, 0, s>>>((const double *)f, P, half, hh, g.dV, out); break;
-    case DVM_F32: k_moments<float><<<grid, t, 0, s>>>((const float *)f, P, half, hh, g.dV, out); break;
-    case DVM_BF16:
-        k_moments<__nv_bfloat16><<<grid, t, 0, s>>>((const __nv_bfloat16 *)f, P, half, hh, g.dV, out);
-        break;
+    case DVM_F64: return moments_t<double>(f, ncells, g, out, s);
+    case DVM_F32: return moments_t<float>(f, ncells, g, out, s);
+    case DVM_BF16: return moments_t<__nv_bfloat16>(f, ncells, g, out, s);
     default: return DVM_EINVAL;
     }
-    return last_status();
 }
 
 int launch_to_f64(int prec, const void *src, double *dst, int64_t n, cudaStream_t s)
