@@ -1051,7 +1051,10 @@ __global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_s
                         Bxy[sxy] = KN * a.g * c.g;
                         Axy[sxy] = Bxy[sxy] * (C0 + a.p + c.p);
                     }
-#pragma unroll
+                    // rolled for FP32 and BF16: less of the instruction cache (24^3
+                    // BF16 4.02 -> 3.94 ms, FP32 4.38 -> 4.33); FP64 on small
+                    // grids is 1% faster unrolled
+#pragma unroll (sizeof(TC) == 8 ? 2 : 1)
                     for (int pz = 0; pz < 2; pz++) {
                         TC g[VEC], gp[VEC];
 #pragma unroll
