@@ -1922,11 +1922,13 @@ int dvm_lbm_step(dvm_ctx *c, int nsteps, double dt, double tau)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     p.threads = dvm::lbm_threads(p.ncells, nsm);
+    p.overlap = p.ncells <= (int64_t)nsm * p.threads;
     p.status = c->d_lstatus;
     p.stream = c->stream;
     for (int s = 0; s < nsteps; s++) {
         p.f_in = c->d_lf[c->lcur];
         p.f_out = c->d_lf[c->lcur ^ 1];
+        p.follows = s > 0;
         rc = dvm::launch_lbm(p);
         if (rc) return fail(c, rc, std::string("lattice Boltzmann launch: ") + cudaGetErrorString(cudaGetLastError()));
         c->lcur ^= 1;
