@@ -56,29 +56,40 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
 // sum j_d f, sum j_d^2 f (xi_d = (h_d/2) j_d, j_d odd).  FP64 runs at 1/64 of
 // the FP32 rate here and thirteen FP64 operations a value bound the kernel at
 // 57 GB/s of its read of f, so FP32 and BF16 storage sum exactly in fixed
-// point instead: with M the cell's largest |f| and sigma = 2^k >= 512 M, each
-// value splits without error (the extraction of Rump, Ogita and Oishi, 2008)
-// into a multiple of 2^(k-24), a multiple of 2^(k-39) and a rest of at most
-// 2^(k-39).  A thread's sums of its 32 values of either multiple, with the
-// weights that k_step's partials use (total size below 16 against the split's
-// margin), are exact in FP32 and go into 64-bit integers; the rests are summed
-// in FP32.  What is lost is below 2^-60 of sum |f|, less than FP64 summation
-// loses.  A cell with non-finite values or M outside [2^-86, 2^115] takes FP64
-// sums.
+// point instead: with 2^m above a warp's largest |f|, each of its values splits
+// without error (the extraction of Rump, Ogita and Oishi, 2008) into multiples
+// of u1 = 2^(m-17), u2 = 2^(m-35) and u3 = 2^(m-53) and a rest of at most u3/2.
+// A thread's sums of its 32 values of each multiple, with the weights that
+// k_step's partials use (total size at most 112), stay below 2^24 units, hence
+// exact in FP32, and go into 64-bit integers; the rests (of values below
+// 2^(m-30)) are summed in FP32, in at most 60 additions a value: off by less
+// than 60 2^-24 2^-54 2^m a value, 2^-60 of the warp's sum of |f| at 24^3.  The
+// warps' sums are added in FP64.  Two multiples and the rests in FP32 instead
+// (rests of 2^-30 of the cell's largest value) took 283 us where this takes 295,
+// but were up to 9.5e-13 of sum |f| off on values of that size, FP64 sums
+// 1.1e-15.  A warp with non-finite values or its largest outside [2^-71, 2^115]
+// takes FP64 sums.
 //
-// f is read once from HBM and twice by its thread, for M and for the sums.
+// f is read once from HBM and twice by its thread, for m and for the sums.
 // Cells of up to 56 KB go through shared memory (PIPE): a CTA takes every
-// gridDim-th cell, and each thread copies its own pieces of the next one with
-// cp.async while it sums this one, so that the stream does not stop for the
-// barriers and the FP64 tail of a cell.  Larger cells are read from memory
-// twice.  17,680 cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 319 us
-// with the cell held in registers (one cell per CTA), 283 us through
-// shared memory; what bounds it now is the arithmetic of the split at 14 warps
-// an SM.
-constexpr int MOM_T = 256;
+// gridDim-th cell by bulk copies, two at a time.  With SPLIT a last warp
+// finishes the cells (FP64, a long serial chain) and refills their buffers while
+// the others go on; CTAs of one or two working warps would lose a third to half
+// of an SM's warps to that and have warp 0 do it (8^3: 123 us the call, 136 with
+// it; 24^3: 399 and 371).  Larger cells are read from memory twice.  17,680
+// cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 295 us now; what bounds
+// it is the arithmetic of the split, about 800 instructions for a warp's 1,024
+// values at 54% of the issue slots.
+constexpr int MOM_T = 224;
 constexpr size_t MOM_ROW = 56 * 1024;
 
-__device__ inline uint32_t abs_bits(float2 v) { return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu); }
+// the largest of |a|, |b|, |c|, NaN if one is
+__device__ inline float max_abs(float a, float b, float c)
+{
+    float m;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
 
 // the seven base sums of a quad at one level of the split, times 2^-quantum
 // as integers: S, X, Y, Z over the four positions, sum e Z_e, sum e S_e,
@@ -88,18 +99,20 @@ __device__ inline void base_sums(const float2 (&a)[8], const float2 (&b)[8], flo
     float2 Sa, Xa, Ya, Za, Sb, Xb, Yb, Zb;
     group_sums(a, Sa, Xa, Ya, Za);
     group_sums(b, Sb, Xb, Yb, Zb);
-    s[0] = (Sa.x + Sa.y) + (Sb.x + Sb.y);
-    s[1] = (Xa.x + Xa.y) + (Xb.x + Xb.y);
-    s[2] = (Ya.x + Ya.y) + (Yb.x + Yb.y);
-    s[3] = (Za.x + Za.y) + (Zb.x + Zb.y);
+    const float2 St = f2_add(Sa, Sb), Xt = f2_add(Xa, Xb), Yt = f2_add(Ya, Yb), Zt = f2_add(Za, Zb);
+    s[0] = St.x + St.y;
+    s[1] = Xt.x + Xt.y;
+    s[2] = Yt.x + Yt.y;
+    s[3] = Zt.x + Zt.y;
     s[4] = (Za.y + 2.0f * Zb.x) + 3.0f * Zb.y;
     s[5] = (Sa.y + 2.0f * Sb.x) + 3.0f * Sb.y;
     s[6] = (Sa.y + 4.0f * Sb.x) + 9.0f * Sb.y;
 }
 
 // the seven weighted sums from the base sums (j = j0 + 2 e along z)
-template <typename T, typename J> __device__ inline void weighted_sums(const T (&s)[7], J jx, J jy, J jz, T (&m)[7])
+template <typename T> __device__ inline void weighted_sums(const T (&s)[7], T jx, T jy, T jz, T (&m)[7])
 {
+    using J = T;
     m[0] += s[0];
     m[1] += s[1] * jx;
     m[2] += s[2] * jy;
@@ -109,8 +122,30 @@ template <typename T, typename J> __device__ inline void weighted_sums(const T (
     m[6] += s[0] * (jz * jz) + s[5] * (J)(4 * jz) + s[6] * (J)4;
 }
 
-// split a thread's 32 values at one level: x = q + r, q a multiple of
-// sigma 2^-24
+// 1.5 2^(e - 127): an x of at most 2^(e - 128) splits against it into a multiple
+// of 2^(e - 150) and a rest of at most half of that
+__device__ inline float sigma_of(int e) { return __int_as_float((e << 23) | 0x400000); }
+
+// the same in integers, times k: one 32 x 32 + 64 bit multiply-add a term (left
+// to the compiler the call of 17,680 cells x 24^3 takes 750 us, so 737)
+__device__ inline void weighted_sums(const int (&s)[7], int jx, int jy, int jz, int k, int64_t (&m)[7])
+{
+    auto add = [&](int i, int v, int w) {
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(m[i]) : "r"(v), "r"(w * k));
+    };
+    add(0, s[0], 1);
+    add(1, s[1], jx);
+    add(2, s[2], jy);
+    add(3, s[3], jz);
+    add(3, s[4], 2);
+    add(4, s[0], jx * jx);
+    add(5, s[0], jy * jy);
+    add(6, s[0], jz * jz);
+    add(6, s[5], 4 * jz);
+    add(6, s[6], 4);
+}
+
+// split a thread's 32 values at one level: x = q + r
 __device__ inline void extract8(float2 (&x)[8], float sigma, float2 (&q)[8])
 {
     const float2 s2 = make_float2(sigma, sigma);
@@ -122,34 +157,50 @@ __device__ inline void extract8(float2 (&x)[8], float sigma, float2 (&q)[8])
 }
 
 struct MomSum {
-    int64_t I[7];  // in units of 2^(k-39)
+    int64_t hi[7], lo[7];  // in units of u1 and u3
     float R[7];
 };
 
-__device__ inline void add_quad(const QV<float> (&x)[8], int ex, int jx, int jy, int jz, MomSum &m)
+__device__ inline uint32_t any_bits(const float2 (&a)[8], const float2 (&b)[8])
 {
-    const float sg1 = __int_as_float((ex + 10) << 23), sg2 = __int_as_float((ex - 5) << 23);  // 2^k, 2^(k-15)
-    const float c1 = __int_as_float((268 - ex) << 23), c2 = __int_as_float((283 - ex) << 23);  // 2^(24-k), 2^(39-k)
+    uint32_t v = 0;
+#pragma unroll
+    for (int o = 0; o < 8; o++)
+        v |= __float_as_uint(a[o].x) | __float_as_uint(a[o].y) | __float_as_uint(b[o].x) | __float_as_uint(b[o].y);
+    return v & 0x7fffffffu;
+}
+
+// m = ex - 126; COARSE: values of 8 significant bits (BF16)
+template <bool COARSE> __device__ inline void add_quad(const QV<float> (&x)[8], int ex, int jx, int jy, int jz, MomSum &m)
+{
     float2 ra[8], rb[8], qa[8], qb[8];
 #pragma unroll
     for (int o = 0; o < 8; o++) {
         ra[o] = x[o].a;
         rb[o] = x[o].b;
     }
-    float s1[7], s2[7], s3[7];
-    extract8(ra, sg1, qa);
-    extract8(rb, sg1, qb);
-    base_sums(qa, qb, s1);
-    extract8(ra, sg2, qa);
-    extract8(rb, sg2, qb);
-    base_sums(qa, qb, s2);
-    base_sums(ra, rb, s3);
-    int64_t v[7];
+    float s[7];
+    int v[7];
+    // the sums of the multiples of 2^(e - 150), in those units
+    auto level = [&](int e) {
+        const float sg = sigma_of(e), c = __int_as_float((277 - e) << 23);
+        extract8(ra, sg, qa);
+        extract8(rb, sg, qb);
+        base_sums(qa, qb, s);
 #pragma unroll
-    for (int k = 0; k < 7; k++)
-        v[k] = (int64_t)__float2int_rn(s1[k] * c1) * 32768 + (int64_t)__float2int_rn(s2[k] * c2);
-    weighted_sums<int64_t, int>(v, jx, jy, jz, m.I);
-    weighted_sums<float, float>(s3, (float)jx, (float)jy, (float)jz, m.R);
+        for (int k = 0; k < 7; k++) v[k] = __float2int_rn(s[k] * c);
+    };
+    level(ex + 7);
+    weighted_sums(v, jx, jy, jz, 1, m.hi);
+    level(ex - 11);
+    weighted_sums(v, jx, jy, jz, 1 << 18, m.lo);
+    if (COARSE && !any_bits(ra, rb)) return;
+    level(ex - 29);
+    weighted_sums(v, jx, jy, jz, 1, m.lo);
+    if (!COARSE || any_bits(ra, rb)) {
+        base_sums(ra, rb, s);
+        weighted_sums<float>(s, (float)jx, (float)jy, (float)jz, m.R);
+    }
 }
 
 // the same sums in FP64
@@ -178,52 +229,108 @@ template <typename TC> __device__ inline void add_quad_f64(const QV<TC> (&x)[8],
         s[5] += e * S;
         s[6] += e * e * S;
     }
-    weighted_sums<double, double>(s, (double)jx, (double)jy, (double)jz, m);
+    weighted_sums<double>(s, (double)jx, (double)jy, (double)jz, m);
 }
 
-template <typename TS, bool PIPE>
-__global__ void __launch_bounds__(MOM_T, 2)
+// barriers of k_moments: the sums of buffer 0 or 1 are ready
+constexpr int BAR_READY = 1;
+
+template <typename TS, bool PIPE, bool SPLIT>
+__global__ void __launch_bounds__(256, 2)
     k_moments(const TS *__restrict__ f, int64_t ncells, int P, int3 half, double3 hh, double dV, double *__restrict__ out)
 {
     using IO = QIO<TS>;
     using TC = typename Store<TS>::TC;
     constexpr int VEC = Store<TS>::VEC;
-    extern __shared__ __align__(16) unsigned char mom_tile[];  // PIPE: [2][8 P]
-    __shared__ uint32_t wmax[MOM_T / 32];
-    __shared__ double red[MOM_T / 32][7];
-    __shared__ int64_t redI[MOM_T / 32][7];
-    __shared__ float redR[MOM_T / 32][7];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, nw = T >> 5, Q = P / VEC;
+    // a cell's sums by warp, in one of two buffers
+    union Red {
+        struct {
+            int64_t hi, lo;
+            float R;
+        } fx;
+        double d;
+    };
+    extern __shared__ __align__(128) unsigned char mom_tile[];  // PIPE: [2][8 P]
+    __shared__ Red red[2][MOM_T / 32][7];
+    __shared__ int rexp[2][MOM_T / 32];  // exponent of the warp's largest value, 0: FP64 sums
+    __shared__ __align__(8) uint64_t full[2], taken[2];  // the cell has arrived; its sums have been read
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x - (SPLIT ? 32 : 0), nw = T >> 5,
+              Q = P / VEC;
     TS *tile = reinterpret_cast<TS *>(mom_tile);
-    // the thread's pieces of cell c into buffer b (each thread reads back only
-    // what it copied)
     auto copy = [&](int64_t c, int b) {
-        if (c < ncells)
-            for (int q = tid; q < Q; q += T)
-#pragma unroll
-                for (int o = 0; o < 8; o++) {
-                    const TS *src = f + (c * 8 + o) * (int64_t)P + q * VEC;
-                    TS *dst = tile + (size_t)(b * 8 + o) * P + q * VEC;
-                    if constexpr (sizeof(TS) == 2) cp_async8(dst, src, 0u);
-                    else cp_async16(dst, src, 0u);
-                }
-        cp_async_commit();
-    };
-    auto nodes = [&](int q, int &jx, int &jy, int &jz) {
-        const int p = q * VEC, t = p / half.z;
-        jz = 2 * (p - t * half.z) + 1;
-        jy = 2 * (t % half.y) + 1;
-        jx = 2 * (t / half.y) + 1;
-    };
-    if constexpr (PIPE) copy(blockIdx.x, 0);
-    int buf = 0;
-    for (int64_t c = blockIdx.x; c < ncells; c += gridDim.x, buf ^= 1) {
-        if constexpr (PIPE) {
-            // the other buffer's values were all used before this cell's
-            // predecessor reached its barriers
-            copy(c + gridDim.x, buf ^ 1);
-            cp_async_wait<1>();
+        if (PIPE && c < ncells) {
+            const uint32_t bytes = 8u * (uint32_t)P * (uint32_t)sizeof(TS);
+            mbar_expect_tx(&full[b], bytes);
+            bulk_g2s(tile + (size_t)b * 8 * P, f + c * 8 * (int64_t)P, bytes, &full[b]);
         }
+    };
+    // one warp: the moments of cell c from the warps' sums
+    auto finish = [&](int64_t c, int b) {
+        // all are through with the cell: the one after next takes its place
+        if (lane == 0) copy(c + 2 * (int64_t)gridDim.x, b);
+        const int k = lane % 7;  // lane: sum k of every fourth warp (lanes 28..31: spare)
+        double s = 0.0;
+        for (int w = lane < 28 ? lane / 7 : nw; w < nw; w += 4) {
+            const int ex = rexp[b][w];
+            const Red &r = red[b][w][k];
+            if (ex == 0) {
+                s += r.d;
+            } else {
+                const double u1 = __longlong_as_double((long long)(1023 + ex - 143) << 52);
+                s += fma((double)r.fx.hi, u1, fma((double)r.fx.lo, u1 * 0x1p-36, (double)r.fx.R));
+            }
+        }
+        __syncwarp();
+        if (SPLIT && lane == 0) mbar_arrive(&taken[b]);
+        s += __shfl_down_sync(0xffffffffu, s, 14);
+        s += __shfl_down_sync(0xffffffffu, s, 7);
+        // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
+        const double s0 = __shfl_sync(0xffffffffu, s, 0);
+        const int d = (lane + 2) % 3;
+        const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
+        const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
+        const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
+        const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
+                     uz2 = __shfl_sync(0xffffffffu, u2, 3);
+        const double ex2 = __shfl_sync(0xffffffffu, e2, 1), ey2 = __shfl_sync(0xffffffffu, e2, 2),
+                     ez2 = __shfl_sync(0xffffffffu, e2, 3);
+        double *o = out + c * 5;
+        if (lane == 0) {
+            o[0] = s0 * dV;
+            o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
+        } else if (lane < 4) {
+            o[lane] = v;
+        }
+    };
+    if (tid == 0) {
+        mbar_init(&taken[0], 1);
+        mbar_init(&taken[1], 1);
+        mbar_init(&full[0], 1);
+        mbar_init(&full[1], 1);
+        mbar_fence_init();
+        copy(blockIdx.x, 0);
+        copy((int64_t)blockIdx.x + gridDim.x, 1);
+    }
+    __syncthreads();
+    if (SPLIT && warp == nw) {
+        int buf = 0;
+        for (int64_t c = blockIdx.x; c < ncells; c += gridDim.x, buf ^= 1) {
+            bar_sync_n(BAR_READY + buf, T + 32);
+            finish(c, buf);
+        }
+        return;
+    }
+    auto node = [&](int q) {
+        const int p = q * VEC, t = p / half.z;
+        return make_int3(2 * (t / half.y) + 1, 2 * (t % half.y) + 1, 2 * (p - t * half.z) + 1);
+    };
+    const int3 j0 = node(tid), j1 = node(tid + T);  // most grids have no more quads a thread
+    int buf = 0, done = 0;
+    for (int64_t c = blockIdx.x; c < ncells; c += gridDim.x, buf ^= 1, done++) {
+        bool here = true;
+        // (waited for twice at most, to leave no copy in flight behind)
+        if constexpr (PIPE)
+            here = mbar_wait(&full[buf], (uint32_t)(done >> 1) & 1u) || mbar_wait(&full[buf], (uint32_t)(done >> 1) & 1u);
         auto load = [&](int q, QV<TC> (&x)[8]) {
 #pragma unroll
             for (int o = 0; o < 8; o++) {
@@ -231,89 +338,68 @@ __global__ void __launch_bounds__(MOM_T, 2)
                 else x[o] = IO::ldg(f + (c * 8 + o) * (int64_t)P + q * VEC);
             }
         };
-        int jx, jy, jz;
-        bool wide = true;  // FP64 sums
+        auto place = [&](int q) {
+            if (PIPE && q < 2 * T) return q == tid ? j0 : j1;
+            return node(q);
+        };
         int ex = 0;
+        MomSum m{};
         if constexpr (sizeof(TC) == 4) {
-            uint32_t mx = 0;
+            float top = 0.0f;
             for (int q = tid; q < Q; q += T) {
                 QV<float> x[8];
                 load(q, x);
 #pragma unroll
-                for (int o = 0; o < 8; o++) mx = max(mx, max(abs_bits(x[o].a), abs_bits(x[o].b)));
+                for (int o = 0; o < 8; o++)
+                    top = max_abs(max_abs(top, x[o].a.x, x[o].a.y), x[o].b.x, x[o].b.y);
             }
-            mx = __reduce_max_sync(0xffffffffu, mx);
-            if (lane == 0) wmax[warp] = mx;
-            __syncthreads();
-            for (int w = 0; w < nw; w++) mx = max(mx, wmax[w]);
-            ex = (int)(mx >> 23);  // M < 2^(ex - 126)
-            wide = ex < 40 || ex > 240;
-            if (!wide) {
-                MomSum m{};
+            ex = (int)(__reduce_max_sync(0xffffffffu, __float_as_uint(top)) >> 23);
+            if (ex < 56 || ex > 240) ex = 0;
+            if (ex) {
 #pragma unroll 1
                 for (int q = tid; q < Q; q += T) {
                     QV<float> x[8];
                     load(q, x);
-                    nodes(q, jx, jy, jz);
-                    add_quad(x, ex, jx, jy, jz, m);
-                }
-                const int64_t I = warp_reduce7<int64_t>(m.I, lane);
-                const float R = warp_reduce7<float>(m.R, lane);
-                if ((lane & 3) == 0 && lane < 28) {
-                    redI[warp][lane >> 2] = I;
-                    redR[warp][lane >> 2] = R;
+                    const int3 j = place(q);
+                    add_quad<sizeof(TS) == 2>(x, ex, j.x, j.y, j.z, m);
                 }
             }
         }
-        if (wide) {
-            double m[7] = {0, 0, 0, 0, 0, 0, 0};
+        double md[7] = {0, 0, 0, 0, 0, 0, 0};
+        if (!ex) {
 #pragma unroll 1
             for (int q = tid; q < Q; q += T) {
                 QV<TC> x[8];
                 load(q, x);
-                nodes(q, jx, jy, jz);
-                add_quad_f64<TC>(x, jx, jy, jz, m);
-            }
-            const double t = warp_reduce7<double>(m, lane);
-            if ((lane & 3) == 0 && lane < 28) red[warp][lane >> 2] = t;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            double s = 0.0;
-            if (lane < 7) {
-                if (wide) {
-                    for (int w = 0; w < nw; w++) s += red[w][lane];
-                } else {
-                    int64_t I = 0;
-                    float R = 0.0f;
-                    for (int w = 0; w < nw; w++) {
-                        I += redI[w][lane];
-                        R += redR[w][lane];
-                    }
-                    s = (double)I * __longlong_as_double((long long)(1023 + ex - 156) << 52) + (double)R;  // 2^(k-39)
-                }
-            }
-            // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
-            const double s0 = __shfl_sync(0xffffffffu, s, 0);
-            const int d = (lane + 2) % 3;
-            const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
-            const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
-            const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
-            const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
-                         uz2 = __shfl_sync(0xffffffffu, u2, 3);
-            const double ex2 = __shfl_sync(0xffffffffu, e2, 1), ey2 = __shfl_sync(0xffffffffu, e2, 2),
-                         ez2 = __shfl_sync(0xffffffffu, e2, 3);
-            double *o = out + c * 5;
-            if (lane == 0) {
-                o[0] = s0 * dV;
-                o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
-            } else if (lane < 4) {
-                o[lane] = v;
+                const int3 j = place(q);
+                add_quad_f64<TC>(x, j.x, j.y, j.z, md);
             }
         }
-        if (sizeof(TC) == 8) __syncthreads();  // red is read above (FP32: the next cell's first barrier)
+        // the buffer's last sums, of two cells ago, have been taken (a wait that
+        // gave up, here or on the copy, leaves NaN)
+        if (SPLIT && done >= 2) here = mbar_wait(&taken[buf], (uint32_t)((done >> 1) - 1) & 1u) && here;
+        if (!here) {
+            ex = 0;
+            md[0] = nan("");
+        }
+        const bool mine = (lane & 3) == 0 && lane < 28;
+        if (ex) {
+            const int64_t hi = warp_reduce7<int64_t>(m.hi, lane), lo = warp_reduce7<int64_t>(m.lo, lane);
+            const float R = warp_reduce7<float>(m.R, lane);
+            if (mine) red[buf][warp][lane >> 2].fx = {hi, lo, R};
+        } else {
+            const double t = warp_reduce7<double>(md, lane);
+            if (mine) red[buf][warp][lane >> 2].d = t;
+        }
+        if (lane == 0) rexp[buf][warp] = ex;
+        __syncwarp();
+        if constexpr (SPLIT) {
+            bar_arrive_n(BAR_READY + buf, T + 32);
+        } else {
+            __syncthreads();
+            if (warp == 0) finish(c, buf);
+        }
     }
-    if constexpr (PIPE) cp_async_wait_all();
 }
 
 template <typename TS>
@@ -344,29 +430,39 @@ int last_status()
     return cudaGetLastError() == cudaSuccess ? DVM_OK : DVM_ECUDA;
 }
 
+template <typename TS, bool PIPE, bool SPLIT>
+int moments_k(const TS *f, int64_t ncells, const MomGrid &g, int t, double *out, cudaStream_t s)
+{
+    const int P = g.half[0] * g.half[1] * g.half[2];
+    const int3 half = make_int3(g.half[0], g.half[1], g.half[2]);
+    const double3 hh = make_double3(0.5 * g.hv[0], 0.5 * g.hv[1], 0.5 * g.hv[2]);
+    auto kern = k_moments<TS, PIPE, SPLIT>;
+    const size_t dyn = PIPE ? 16 * (size_t)P * sizeof(TS) : 0;
+    int64_t grid = ncells;
+    t += SPLIT ? 32 : 0;
+    if (PIPE) {
+        int dev = 0, nsm = 0, occ = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * MOM_ROW)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, t, dyn) != cudaSuccess || occ < 1)
+            return DVM_ECUDA;
+        grid = std::min<int64_t>(ncells, (int64_t)nsm * occ);
+    }
+    kern<<<(unsigned)grid, t, dyn, s>>>(f, ncells, P, half, hh, g.dV, out);
+    return last_status();
+}
+
 template <typename TS> int moments_t(const void *f, int64_t ncells, const MomGrid &g, double *out, cudaStream_t s)
 {
     const int P = g.half[0] * g.half[1] * g.half[2], Q = P / Store<TS>::VEC;
-    // one quad a thread up to 256 quads, then two or more, evenly (24^3: 432
+    const TS *ft = static_cast<const TS *>(f);
+    // one quad a thread up to MOM_T quads, then two or more, evenly (24^3: 432
     // quads on 224 threads)
     const int rounds = (Q + MOM_T - 1) / MOM_T, t = ((Q + rounds - 1) / rounds + 31) / 32 * 32;
-    const int3 half = make_int3(g.half[0], g.half[1], g.half[2]);
-    const double3 hh = make_double3(0.5 * g.hv[0], 0.5 * g.hv[1], 0.5 * g.hv[2]);
-    const TS *ft = static_cast<const TS *>(f);
-    const size_t row = (size_t)8 * P * sizeof(TS);
-    if (row > MOM_ROW) {
-        k_moments<TS, false><<<(unsigned)ncells, t, 0, s>>>(ft, ncells, P, half, hh, g.dV, out);
-        return last_status();
-    }
-    auto kern = k_moments<TS, true>;
-    int dev = 0, nsm = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * MOM_ROW)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, t, 2 * row) != cudaSuccess || occ < 1)
-        return DVM_ECUDA;
-    kern<<<(unsigned)std::min<int64_t>(ncells, (int64_t)nsm * occ), t, 2 * row, s>>>(ft, ncells, P, half, hh, g.dV, out);
-    return last_status();
+    if ((size_t)8 * P * sizeof(TS) > MOM_ROW) return moments_k<TS, false, false>(ft, ncells, g, t, out, s);
+    if (t >= 96) return moments_k<TS, true, true>(ft, ncells, g, t, out, s);
+    return moments_k<TS, true, false>(ft, ncells, g, t, out, s);
 }
 
 // Row copies between buffers: entry r of rows is {destination buffer, row,

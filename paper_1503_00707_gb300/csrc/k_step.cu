@@ -154,9 +154,6 @@ __device__ inline typename Num<TC>::X split(double v)
     }
 }
 
-__device__ inline void bar_sync_n(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ inline void bar_arrive_n(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-
 // named barriers: BAR_P + j % 4 "partials of cell j ready",
 // BAR_C + j % 4 "coefficients of cell j ready"
 constexpr int BAR_P = 1, BAR_C = 5;
