@@ -17,10 +17,10 @@
 //  k_hs_bc   the same sums one cell at a time, for grids whose pair tiles do
 //            not fit in shared memory twice (more than 14,336 nodes).
 //  k_hs_corr per cell: the five coefficients of P (Eq. 6) from the moment
-//            system, its sums formed exactly in an integer basis and
-//            carried in double-float, solved in FP64 in the centred basis
+//            system, its sums formed in an integer basis to about twice
+//            FP32 precision (hs_sums.cuh), solved in the centred basis
 //            (1, c, |c|^2 - 3), c = (xi - u)/sqrt(T), and refined against
-//            the exact sums; then I = -f P B + C and f <- f + dt/Kn I in
+//            those sums in FP64; then I = -f P B + C and f <- f + dt/Kn I in
 //            place.
 #include <cuda_runtime.h>
 
@@ -32,6 +32,7 @@
 #include "async.cuh"
 #include "common.cuh"
 #include "hs.hpp"
+#include "hs_sums.cuh"
 #include "quads.cuh"
 
 namespace dvm {
@@ -312,82 +313,27 @@ __global__ void __launch_bounds__(HT, 1)
     }
 }
 
-// Sum2 accumulation (Ogita, Rump and Oishi, 2005) of exact products:
-// s + e carries the running sum to about twice the FP32 precision.
-struct Acc2 {
-    float s, e;
-};
-// a += (x + xl) k, with x k split exactly (FMA) and xl k a small correction
-__device__ inline void acc2_prod(Acc2 &a, float x, float xl, float k)
-{
-    const float p = x * k;
-    const float pe = fmaf(x, k, -p);
-    const float s = a.s + p;
-    const float bb = s - a.s;
-    const float se = (a.s - (s - bb)) + (p - bb);
-    a.s = s;
-    a.e += se + fmaf(xl, k, pe);
-}
-
-constexpr int NSUM = 20;  // 15 distinct entries of the moment matrix, 5 gain moments
-
-// The signed sums over the eight sign groups that the moment system needs, per
-// position (packed pairs of z nodes), from the sums p and differences m of the
-// groups' pairs along z: S, X, Y, Z as group_sums, and XY = sum s_x s_y x, XZ,
-// YZ.
-__device__ inline void group_sums7(const float2 (&p)[4], const float2 (&m)[4], float2 (&v)[7])
-{
-    const float2 pp0 = f2_add(p[0], p[1]), pm0 = f2_sub(p[1], p[0]);
-    const float2 pp1 = f2_add(p[2], p[3]), pm1 = f2_sub(p[3], p[2]);
-    v[0] = f2_add(pp0, pp1);
-    v[1] = f2_sub(pp1, pp0);
-    v[2] = f2_add(pm0, pm1);
-    v[4] = f2_sub(pm1, pm0);
-    const float2 mp0 = f2_add(m[0], m[1]), mm0 = f2_sub(m[1], m[0]);
-    const float2 mp1 = f2_add(m[2], m[3]), mm1 = f2_sub(m[3], m[2]);
-    v[3] = f2_add(mp0, mp1);
-    v[5] = f2_sub(mp1, mp0);
-    v[6] = f2_add(mm0, mm1);
-}
-
-// sigma = 2^k > 16 max |x|: the split x = q + r against it, q = fl(fl(x +
-// sigma) - sigma), leaves q a multiple of 2^(k-24) whose signed sums over
-// eight groups are exact in FP32, and |r| <= 2^(k-24)
-__device__ inline float2 split_sigma(const float2 (&x)[8])
-{
-    uint32_t mx = 0;
-#pragma unroll
-    for (int o = 0; o < 8; o++)
-        mx = max(mx, max(__float_as_uint(x[o].x) & 0x7fffffffu, __float_as_uint(x[o].y) & 0x7fffffffu));
-    const int ex = min((int)(mx >> 23), 249);
-    const float sg = __int_as_float((ex + 5) << 23);
-    return make_float2(sg, sg);
-}
-
 // k_hs_corr: one CTA per cell.  The correction polynomial of Eq. 6,
 // P = 1 + d.phi, phi = (1, c, |c|^2 - 3), c = (xi - u)/sqrt(T), makes
 // I = C - f P B conserve mass, momentum and energy.  With xi_d = (h/2) j_d
 // (j_d odd integers, the same h on every axis) the integer basis psi^ = (1,
 // j_x, j_y, j_z, |j|^2) spans the same polynomials, so the 15 sums A^_rs =
 // sum_i psi^_r psi^_s f_i B_i and the 5 sums c^_r = sum_i psi^_r C_i have
-// integer weights below 2^24.  A thread takes two z nodes at one position of
-// all eight sign groups: f B (its product split exactly) and C, split
-// against the 16 values' largest, give the signed sums over the groups as an
-// exact part and a rest of 2^-19 of it, and 20 products of those by integers,
-// split exactly (FMA), go into Sum2 accumulators: 22 operations a node where a
-// node at a time takes 72.  One thread solves A^ e = c^, e = (1, 0, 0, 0, 0) +
-// L^T d (L the map psi^ -> phi), in FP64: the factor of L A^ L^T (well
-// conditioned), refined twice against the residual of the sums.  That
-// residual, sum_i psi_r I_i dV with psi = (1, xi, |xi|^2), goes to res (may be
-// null).  Then I_i is evaluated in FP32 with the FP32 copy of d and
-// f <- f + dt/Kn I (or I to q_out).
+// integer weights.  A thread takes two z nodes at one position of all eight
+// sign groups (hs_sums.cuh): about 30 operations a node where a node at a time
+// takes 72, at the same precision (3e-15 of the terms' sizes at worst, rms 6e-16).
+// The lanes of warp 0 solve A^ e = c^, e = (1, 0, 0, 0, 0) + L^T d (L the map
+// psi^ -> phi), through the well-conditioned L A^ L^T, refined against FP64
+// residuals of the sums.  The last residual, sum_i psi_r I_i dV with
+// psi = (1, xi, |xi|^2), goes to res (may be null).  Then I_i is evaluated in
+// FP32 with the FP32 copy of d and f <- f + dt/Kn I (or I to q_out).
 // Bound by HBM at best (f, B, C in, f out); 12,016 cells x 24^3 (2.66 GB):
 // 1.81 -> 0.87 ms, 16,584 x 16^3 0.94 -> 0.53 ms (a node at a time, FP64 factor,
 // 256 threads before); what is left is the serial solve and the sums' reduction
 // per cell.
 // five CTAs of 128 threads per SM (96 registers): four other cells' passes
-// overlap one cell's serial solve (whole steps at 16^3 / 24^3: 3.53 / 7.80 ms;
-// 6 x 128 3.56 / 8.00, 12 x 64 3.59 / 8.05, 3 x 256 3.74 / 7.93)
+// overlap one cell's serial solve (whole steps at 16^3 / 24^3: 3.42 / 7.65 ms;
+// 4 x 128 without spills 3.48 / 7.66)
 __global__ void __launch_bounds__(CT, 5)
     k_hs_corr(float *__restrict__ f, const float *__restrict__ Bp, const float *__restrict__ Cp,
               const float *__restrict__ xi3, double hh, double dV, const double *__restrict__ mom, int nv, int3 half,
@@ -416,93 +362,42 @@ __global__ void __launch_bounds__(CT, 5)
     float *fc = f + cell * (int64_t)nv;
     const float *Bc = Bp + row * (int64_t)nv, *Cc = Cp + row * (int64_t)nv;
     auto ld2 = [](const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); };
-    // The entries are numbered as the upper triangle of the 5x5 matrix over
-    // (1, j_x, j_y, j_z, |j|^2), then the 5 right-hand sums.
+    auto node = [&](int p, float &a, float &b, float &c) {
+        const int t = p / hz;
+        a = (float)(2 * (t / half.y) + 1);
+        b = (float)(2 * (t % half.y) + 1);
+        c = (float)(2 * (p - t * hz) + 1);
+    };
     Acc2 acc[NSUM];
 #pragma unroll
     for (int k = 0; k < NSUM; k++) acc[k] = Acc2{0.0f, 0.0f};
 #pragma unroll 1
     for (int p = 2 * tid; p < P; p += 2 * T) {
-        const int t = p / hz;
-        const float a = (float)(2 * (t / half.y) + 1), b = (float)(2 * (t % half.y) + 1);
-        const float c0 = (float)(2 * (p - t * hz) + 1);
-        float2 w[8], wl[8], V[7], Vr[7];
+        float a, b, c0;
+        node(p, a, b, c0);
+        float2 w[8], wl[8];
 #pragma unroll
         for (int o = 0; o < 8; o++) {
             w[o] = *reinterpret_cast<const float2 *>(fc + o * P + p);
             wl[o] = ld2(Bc + o * P + p);
         }
-#pragma unroll
-        for (int o = 0; o < 8; o++) {
-            // f B = w + wl exactly
-            const float2 m = __fmul2_rn(w[o], wl[o]);
-            wl[o] = __ffma2_rn(w[o], wl[o], make_float2(-m.x, -m.y));
-            w[o] = m;
-        }
-        // the sums of x + xl over the groups: exact part to V, rest to Vr
-        auto sums = [&](const float2 (&x)[8], const float2 *xl) {
-            const float2 sg = split_sigma(x);
-            float2 qp[4], qm[4], rp[4], rm[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const float2 q0 = f2_sub(f2_add(x[2 * k], sg), sg), q1 = f2_sub(f2_add(x[2 * k + 1], sg), sg);
-                float2 r0 = f2_sub(x[2 * k], q0), r1 = f2_sub(x[2 * k + 1], q1);
-                if (xl) {
-                    r0 = f2_add(r0, xl[2 * k]);
-                    r1 = f2_add(r1, xl[2 * k + 1]);
-                }
-                qp[k] = f2_add(q0, q1);
-                qm[k] = f2_sub(q1, q0);
-                rp[k] = f2_add(r0, r1);
-                rm[k] = f2_sub(r1, r0);
-            }
-            group_sums7(qp, qm, V);
-            group_sums7(rp, rm, Vr);
-        };
-        sums(w, wl);
-#pragma unroll
-        for (int e = 0; e < 2; e++) {
-            const float cz = c0 + 2.0f * e, j2 = a * a + b * b + cz * cz;
-            auto put = [&](int k, int v, float coef) {
-                acc2_prod(acc[k], e ? V[v].y : V[v].x, e ? Vr[v].y : Vr[v].x, coef);
-            };
-            put(0, 0, 1.0f);          // (1, 1)
-            put(1, 1, a);             // (1, j_x)
-            put(2, 2, b);             // (1, j_y)
-            put(3, 3, cz);            // (1, j_z)
-            put(4, 0, j2);            // (1, |j|^2)
-            put(5, 0, a * a);         // (j_x, j_x)
-            put(6, 4, a * b);         // (j_x, j_y)
-            put(7, 5, a * cz);        // (j_x, j_z)
-            put(8, 1, a * j2);        // (j_x, |j|^2)
-            put(9, 0, b * b);         // (j_y, j_y)
-            put(10, 6, b * cz);       // (j_y, j_z)
-            put(11, 2, b * j2);       // (j_y, |j|^2)
-            put(12, 0, cz * cz);      // (j_z, j_z)
-            put(13, 3, cz * j2);      // (j_z, |j|^2)
-            put(14, 0, j2 * j2);      // (|j|^2, |j|^2)
-        }
+        add_losses(acc, w, wl, a, b, c0);
+    }
+    // (a loop of its own: fewer accumulators at a time in registers)
+#pragma unroll 1
+    for (int p = 2 * tid; p < P; p += 2 * T) {
+        float a, b, c0;
+        node(p, a, b, c0);
+        float2 w[8];
 #pragma unroll
         for (int o = 0; o < 8; o++) w[o] = ld2(Cc + o * P + p);
-        sums(w, nullptr);
-#pragma unroll
-        for (int e = 0; e < 2; e++) {
-            const float cz = c0 + 2.0f * e, j2 = a * a + b * b + cz * cz;
-            auto put = [&](int k, int v, float coef) {
-                acc2_prod(acc[k], e ? V[v].y : V[v].x, e ? Vr[v].y : Vr[v].x, coef);
-            };
-            put(15, 0, 1.0f);
-            put(16, 1, a);
-            put(17, 2, b);
-            put(18, 3, cz);
-            put(19, 0, j2);
-        }
+        add_gains(acc, w, a, b, c0);
     }
 #pragma unroll
     for (int k = 0; k < NSUM; k++) {
-        const float s = acc[k].s + acc[k].e;
-        const float bb = s - acc[k].s;
-        part[k][tid] = ffn{s, (acc[k].s - (s - bb)) + (acc[k].e - bb)};
+        float lo;
+        const float hi = two_sum(acc[k].s, acc[k].e, lo);
+        part[k][tid] = ffn{hi, lo};
     }
     __syncthreads();
     // the warps take the sums in turn and add each over the CTA in double-float

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "f2.cuh"
+
 namespace dvm {
 
 // The values one thread handles per group: four FP32 values as two packed
@@ -122,10 +124,6 @@ template <typename TC> __device__ inline TC warp_reduce7(const TC (&m)[7], int l
     c += __shfl_xor_sync(0xffffffffu, c, 1);
     return c;
 }
-
-__device__ inline float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-// b - a, rounded once
-__device__ inline float2 f2_sub(float2 b, float2 a) { return __ffma2_rn(a, make_float2(-1.0f, -1.0f), b); }
 
 // Signed sums over the eight sign groups, per position (packed pairs):
 // S = sum_o x_o and X, Y, Z = sum_o s_d(o) x_o with s_d = +1 in the groups of
