@@ -590,10 +590,8 @@ void hs_free(HsTables &t, const DevFree &dfree)
     if (t.d_lane) dfree(t.d_lane);
     if (t.d_desc) dfree(t.d_desc);
     if (t.d_bc) dfree(t.d_bc);
-    if (t.d_pair) dfree(t.d_pair);
     t.d_tab = t.d_lane = nullptr;
     t.d_desc = nullptr;
-    t.d_pair = nullptr;
     t.chunks = 0;
     t.prep_cells = 0;
     t.d_idx = nullptr;

@@ -31,10 +31,9 @@ struct HsTables {
     float *d_xi = nullptr;            // node velocities [3][nv], FP32
     double hh = 0.0;                  // half the velocity spacing (the same on every axis)
     int half[3] = {0, 0, 0};          // nodes per axis / 2 (the grid's sign-group shape)
-    // scratch for bc_cells cells at a time: B and C, [2][bc_cells][nv], and f
+    // scratch for bc_cells cells at a time: B and C, [2][bc_cells][nv], then f
     // as pairs of cells, [bc_cells / 2][nv][2] (packed tables)
     float *d_bc = nullptr;
-    float *d_pair = nullptr;
     int64_t prep_cells = 0;           // the mesh size the scratch was made for
     int64_t bc_cells = 0;
 };

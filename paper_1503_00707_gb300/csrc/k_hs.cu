@@ -584,13 +584,12 @@ int hs_prepare(HsTables &t, int64_t ncells, const DevAlloc &alloc, const DevFree
     if (!t.ready) return DVM_ESTATE;
     if (t.d_bc && t.prep_cells == ncells) return DVM_OK;
     if (t.d_bc) dfree(t.d_bc);
-    if (t.d_pair) dfree(t.d_pair);
-    t.d_bc = t.d_pair = nullptr;
     t.prep_cells = 0;
     t.bc_cells = batch_rows(ncells, t.nv, (size_t)4 << 30);
-    t.d_bc = static_cast<float *>(alloc((size_t)t.bc_cells * t.nv * 2 * sizeof(float)));
-    if (t.chunks) t.d_pair = static_cast<float *>(alloc((size_t)t.bc_cells * t.nv * sizeof(float)));
-    if (!t.d_bc || (t.chunks && !t.d_pair)) return DVM_ENOMEM;
+    // one block (an allocation can cost a first step more than a small mesh's
+    // kernels): B, C and, for the pair kernel, f as pairs
+    t.d_bc = static_cast<float *>(alloc((size_t)t.bc_cells * t.nv * (t.chunks ? 3 : 2) * sizeof(float)));
+    if (!t.d_bc) return DVM_ENOMEM;
     t.prep_cells = ncells;
     return DVM_OK;
 }
@@ -717,7 +716,7 @@ int launch_hs_general(HsTables &t, const StepParams &p, float *f, const int32_t 
     const int rc = bc_plan(t, p.nv, t.bc_cells, L);
     if (rc) return rc;
     const CorrArgs c{p.dV, p.mom_out, q_out ? 0.0f : (float)(dt / kn), q_out, q_out ? nullptr : p.res_out};
-    return run_batches(L, t, f, t.d_bc, t.d_pair, p.nv, p.ncells, list, count, c, p.stream, p.status);
+    return run_batches(L, t, f, t.d_bc, t.d_bc + 2 * t.bc_cells * p.nv, p.nv, p.ncells, list, count, c, p.stream, p.status);
 }
 
 // ---------------------------------------------------------------- allocation-free variant
