@@ -285,6 +285,17 @@ int upload_freestream(dvm_ctx *c)
     return rc;
 }
 
+// The network's work buffers of these sets for n rows.
+int mlp_reserve_sets(dvm_ctx *c, std::initializer_list<int> sets, int64_t n)
+{
+    for (int k : sets) {
+        const int rc = dvm::mlp_reserve(c->mlp, k, n, [c](size_t b) { return dev_alloc(c, b); },
+                                        [c](void *p) { dev_free(c, p); });
+        if (rc) return fail(c, rc, "device allocation (network work buffers)");
+    }
+    return DVM_OK;
+}
+
 // Buffers of the learned collision for the current mesh, the sensor
 // stencil, and network work space for one row per cell.
 int learned_prepare(dvm_ctx *c)
@@ -323,8 +334,8 @@ int learned_prepare(dvm_ctx *c)
     }
     int rc = DVM_OK;
     if (c->mlp_set) {
-        rc = dvm::mlp_reserve(c->mlp, 2 * nc, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
-        if (rc) return fail(c, rc, "device allocation (network work buffers)");
+        rc = mlp_reserve_sets(c, {dvm::MLP_FORWARD}, 2 * nc);
+        if (rc) return rc;
     }
     rc = dvm::hs_prepare(c->hs, nc, [c](size_t b) { return dev_alloc(c, b); }, [c](void *q) { void *r = q; dev_free(c, r); });
     return rc ? fail(c, rc, "hard-sphere scratch allocation failed") : DVM_OK;
@@ -1527,8 +1538,8 @@ int dvm_mlp_forward(dvm_ctx *c, const float *x, int64_t n, float *y)
 {
     if (!c || !x || !y || n < 1) return DVM_EINVAL;
     if (!c->mlp_set) return fail(c, DVM_ESTATE, "no weights set");
-    int rc = dvm::mlp_reserve(c->mlp, n, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
-    if (rc) return fail(c, rc, "device allocation (network work buffers)");
+    int rc = mlp_reserve_sets(c, {dvm::MLP_FORWARD, dvm::MLP_HOST_ROWS}, n);
+    if (rc) return rc;
     float *dx = c->mlp.rows(0), *dy = c->mlp.rows(1);
     rc = cuda_check(c, cudaMemcpyAsync(dx, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
     if (!rc) rc = dvm::mlp_forward(c->mlp, dx, n, dy, c->d_status, c->stream);
@@ -1541,8 +1552,8 @@ int dvm_mlp_loss_grad(dvm_ctx *c, const float *x, const float *t, int64_t n, flo
 {
     if (!c || !x || !t || n < 1) return DVM_EINVAL;
     if (!c->mlp_set) return fail(c, DVM_ESTATE, "no weights set");
-    int rc = dvm::mlp_reserve(c->mlp, n, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
-    if (rc) return fail(c, rc, "device allocation (network work buffers)");
+    int rc = mlp_reserve_sets(c, {dvm::MLP_FORWARD, dvm::MLP_GRAD, dvm::MLP_HOST_ROWS}, n);
+    if (rc) return rc;
     float *dx = c->mlp.rows(0), *dt = c->mlp.rows(1);
     rc = cuda_check(c, cudaMemcpyAsync(dx, x, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy x");
     if (!rc) rc = cuda_check(c, cudaMemcpyAsync(dt, t, (size_t)n * 256, cudaMemcpyHostToDevice, c->stream), "copy t");
@@ -1562,8 +1573,8 @@ int dvm_learned_train(dvm_ctx *c, const float *x, const float *t, int64_t n, int
     if (!c || !x || !t || n < 1 || epochs < 1 || batch < 1 || !(lr > 0.0)) return DVM_EINVAL;
     if (!c->mlp_set) return fail(c, DVM_ESTATE, "no weights set");
     const int64_t nb = std::min<int64_t>(batch, n);
-    int rc = dvm::mlp_reserve(c->mlp, nb, [c](size_t b) { return dev_alloc(c, b); }, [c](void *p) { void *q = p; dev_free(c, q); });
-    if (rc) return fail(c, rc, "device allocation (network work buffers)");
+    int rc = mlp_reserve_sets(c, {dvm::MLP_FORWARD, dvm::MLP_GRAD}, nb);
+    if (rc) return rc;
     DevArr dx(c, (size_t)n * 256), dt(c, (size_t)n * 256);
     if (!dx.p || !dt.p) return fail(c, DVM_ENOMEM, "device allocation (training rows)");
     std::vector<int64_t> perm(n);

@@ -442,6 +442,7 @@ void mlp_free(Mlp &m, const DevFreeF &dfree)
     m.loss = nullptr;
     m.ready = false;
     for (auto &b : m.work) b.reset(dfree);
+    for (auto &c : m.cap) c = 0;
 }
 
 int mlp_cast(Mlp &m, cudaStream_t s)
@@ -466,29 +467,31 @@ const float *mlp_bias(const Mlp &m, int l) { return m.w + param_offset(l) + (siz
 // pipelined loads takes 0.26 ms more at 30,000 rows than 21 splits.
 static int wgrad_splits(int64_t n) { return n <= 12000 ? (int)std::min<int64_t>(21, (n + 63) / 64) : 1; }
 
-// working buffers for a batch of n rows (n padded to a multiple of 64)
-int mlp_reserve(Mlp &m, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree)
+// one set of working buffers for a batch of n rows (n padded to a multiple of 64)
+int mlp_reserve(Mlp &m, int set, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree)
 {
     const int64_t np = (n + 63) / 64 * 64;
-    if (np <= m.cap) return DVM_OK;
-    for (auto &b : m.work) b.reset(dfree);
-    m.cap = 0;
+    if (np <= m.cap[set]) return DVM_OK;
     const size_t tiles = (size_t)(np + 127) / 128;
-    const size_t sz[] = {(size_t)np * 64 * 2, (size_t)np * 64 * 2,           // X, Xt
+    const size_t sz[] = {(size_t)np * 64 * 2, (size_t)np * 256 * 2 * 3,      // X, H
+                         (size_t)np * 64 * 2,                                // Xt
                          (size_t)np * 256 * 4 * 3,                           // Z1..Z3
-                         (size_t)np * 256 * 2 * 3, (size_t)np * 256 * 2 * 3, // H, Ht
+                         (size_t)np * 256 * 2 * 3,                           // Ht
                          (size_t)np * 64 * 2, (size_t)np * 64 * 2,           // dO, dOt
                          (size_t)np * 256 * 2 * 2, (size_t)np * 256 * 2 * 3, // dZ (two in turn), dZt of each layer
                          (size_t)21 * MLP_NPARAM * 4,                        // partial weight gradients (at most 21 splits)
                          tiles * 832 * 4, tiles * 8,                         // partial bias gradients and losses
                          (size_t)np * 256, (size_t)np * 256};                // a host call's rows
     static_assert(sizeof(sz) / sizeof(sz[0]) == MLP_NWORK, "work buffer count");
-    for (int i = 0; i < MLP_NWORK; i++) {
+    const int first[MLP_NSETS + 1] = {W_X, W_XT, W_R0, MLP_NWORK};
+    for (int i = first[set]; i < first[set + 1]; i++) m.work[i].reset(dfree);
+    m.cap[set] = 0;
+    for (int i = first[set]; i < first[set + 1]; i++) {
         m.work[i].p = alloc(sz[i]);
         m.work[i].bytes = sz[i];
         if (!m.work[i].p) return DVM_ENOMEM;
     }
-    m.cap = np;
+    m.cap[set] = np;
     return DVM_OK;
 }
 
@@ -496,7 +499,7 @@ int mlp_reserve(Mlp &m, int64_t n, const DevAllocF &alloc, const DevFreeF &dfree
 // keeps pre-activations and transposed activations for the backward pass
 static int forward3(Mlp &m, int64_t n, bool train, int *status, cudaStream_t s)
 {
-    const int64_t np = m.cap;
+    const int64_t np = m.cap[MLP_FORWARD], nt = m.cap[MLP_GRAD];
     auto *Z = static_cast<float *>(m.work[W_Z].p);
     auto *H = static_cast<__nv_bfloat16 *>(m.work[W_H].p);
     auto *Ht = static_cast<__nv_bfloat16 *>(m.work[W_HT].p);
@@ -511,10 +514,10 @@ static int forward3(Mlp &m, int64_t n, bool train, int *status, cudaStream_t s)
         g.bias = mlp_bias(m, l);
         g.status = status;
         g.act = 1;
-        g.Cf = train ? Z + (size_t)l * np * 256 : nullptr;
+        g.Cf = train ? Z + (size_t)l * nt * 256 : nullptr;
         g.H = H + (size_t)l * np * 256;
-        g.HT = train ? Ht + (size_t)l * np * 256 : nullptr;
-        g.ldt = np;
+        g.HT = train ? Ht + (size_t)l * nt * 256 : nullptr;
+        g.ldt = nt;
         in = g.H;
         int rc = gemm<EP_FORWARD>(g, s);
         if (rc) return rc;
@@ -525,7 +528,7 @@ static int forward3(Mlp &m, int64_t n, bool train, int *status, cudaStream_t s)
 static GemmArgs layer4(Mlp &m, int64_t n, int *status)
 {
     GemmArgs g{};
-    g.A = static_cast<__nv_bfloat16 *>(m.work[W_H].p) + (size_t)2 * m.cap * 256;
+    g.A = static_cast<__nv_bfloat16 *>(m.work[W_H].p) + (size_t)2 * m.cap[MLP_FORWARD] * 256;
     g.B = m.W[3];
     g.lda = g.ldb = g.K = 256;
     g.M = n;
@@ -537,7 +540,7 @@ static GemmArgs layer4(Mlp &m, int64_t n, int *status)
 
 int mlp_forward(Mlp &m, const float *x_dev, int64_t n, float *y_dev, int *status, cudaStream_t s)
 {
-    if (n > m.cap) return DVM_EINVAL;
+    if (n > m.cap[MLP_FORWARD]) return DVM_EINVAL;
     k_to_bf16<<<(unsigned)((n + 63) / 64), 256, 0, s>>>(x_dev, static_cast<__nv_bfloat16 *>(m.work[W_X].p), nullptr, n, 0);
     count_launch();
     int rc = forward3(m, n, false, status, s);
@@ -550,8 +553,8 @@ int mlp_forward(Mlp &m, const float *x_dev, int64_t n, float *y_dev, int *status
 // loss and gradient (m.g) for rows x_dev / targets t_dev (FP32 [n][64])
 int mlp_grad(Mlp &m, const float *x_dev, const float *t_dev, int64_t n, int *status, cudaStream_t s)
 {
-    if (n > m.cap) return DVM_EINVAL;
-    const int64_t np = m.cap;
+    if (n > m.cap[MLP_FORWARD] || n > m.cap[MLP_GRAD]) return DVM_EINVAL;
+    const int64_t np = m.cap[MLP_GRAD];
     const int tiles = (int)((n + 127) / 128), splits = wgrad_splits(n);
     auto *X = static_cast<__nv_bfloat16 *>(m.work[W_X].p);
     auto *Xt = static_cast<__nv_bfloat16 *>(m.work[W_XT].p);
