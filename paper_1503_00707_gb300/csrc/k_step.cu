@@ -666,11 +666,12 @@ __device__ inline int solve_cell(const StepParams &p, StepSmem<TC> &sm, const Co
 
 // PC: the group size P as a compile-time constant (0: read it from p), so
 // that every group offset of the unrolled loops is an immediate.
-// 16^3 grids (192 threads): 96 registers for three CTAs an SM, six solver and
-// twelve compute warps instead of four and eight (27k cells FP32, four steps:
-// 1.40 -> 1.29 ms).
-template <typename TS, int DIM, int COLL, int PC>
-__global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_step(const StepParams p)
+// SMALL: CTAs of three or four compute warps (160 or 192 threads; FP32 and BF16
+// in 3D, for example 16^3): 96 registers for three CTAs an SM, six solver and
+// twelve compute warps instead of four and eight (27k cells x 16^3 FP32, four
+// steps: 1.40 -> 1.29 ms).
+template <typename TS, int DIM, int COLL, int PC, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 192 : MAXT, SMALL ? 3 : 1) k_step(const StepParams p)
 {
     using S = Store<TS>;
     using IO = QIO<TS>;
@@ -955,12 +956,11 @@ __global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_s
             // Cells without further sources take a copy of the loop without
             // their branch, in which the loads of several groups are scheduled
             // together (24^3, 159k cells: BF16 4.39 -> 4.02 ms, FP32 4.41 ->
-            // 4.38).  Three small CTAs an SM (16^3) hide the further sources'
+            // 4.38).  Three small CTAs an SM hide the further sources'
             // latency for one another, and one loop with those added at its
-            // end is the faster form (27k cells, four steps: 1.28 -> 1.18
-            // ms;
-            // at 24^3, where nothing else runs meanwhile, it takes 6.6 ms).
-            if constexpr (PC == 512) {
+            // end is the faster form (27k cells x 16^3, four steps: 1.28 -> 1.18
+            // ms; at 24^3, where nothing else runs meanwhile, it takes 6.6 ms).
+            if constexpr (SMALL) {
                 transport(std::false_type{});
 #pragma unroll 1
                 for (uint32_t m = valid && active ? xm : 0u; m; m &= m - 1) {
@@ -1096,10 +1096,10 @@ __global__ void __launch_bounds__(PC == 512 ? 192 : MAXT, PC == 512 ? 3 : 1) k_s
     cp_async_wait_all();
 }
 
-template <typename TS, int DIM, int COLL, int PC>
+template <typename TS, int DIM, int COLL, int PC, bool SMALL>
 int launch_kernel(const StepParams &p, int ncw)
 {
-    auto kern = k_step<TS, DIM, COLL, PC>;
+    auto kern = k_step<TS, DIM, COLL, PC, SMALL>;
     const int threads = (ncw + 2) * 32;
     const size_t dyn = step_dyn_bytes<TS, DIM>(p.P);
     // the queries below take longer than a small step's launch: made once per
@@ -1129,15 +1129,20 @@ int launch_kernel(const StepParams &p, int ncw)
 }
 
 // compile-time group sizes for the 24^3 and 16^3 grids of 3D FP32/BF16 runs
-// (BGK, entropic BGK and transport alone)
+// (BGK, entropic BGK and transport alone), and the CTAs that take SMALL
 template <typename TS, int DIM, int COLL>
 int launch_sized(const StepParams &p, int ncw)
 {
     if constexpr (DIM == 3 && sizeof(TS) <= 4) {
-        if (p.P == 1728) return launch_kernel<TS, DIM, COLL, 1728>(p, ncw);
-        if (p.P == 512) return launch_kernel<TS, DIM, COLL, 512>(p, ncw);
+        if (p.P == 1728) return launch_kernel<TS, DIM, COLL, 1728, false>(p, ncw);
+        if (p.P == 512) return launch_kernel<TS, DIM, COLL, 512, true>(p, ncw);
+        // three or four compute warps: 27k cells FP32 12 x 20 x 16 337 -> 317 us a
+        // step (entropic 466 -> 380), 12 x 12 x 16 260 -> 248, BF16 382 -> 370 and
+        // 300 -> 294.  One or two, of which more CTAs fit an SM anyway: 8 x 8 x 24
+        // 208 -> 214, BF16 16 x 16 x 8 229 -> 257.
+        if (ncw == 3 || ncw == 4) return launch_kernel<TS, DIM, COLL, 0, true>(p, ncw);
     }
-    return launch_kernel<TS, DIM, COLL, 0>(p, ncw);
+    return launch_kernel<TS, DIM, COLL, 0, false>(p, ncw);
 }
 
 template <typename TS, int DIM>
