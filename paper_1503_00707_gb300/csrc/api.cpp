@@ -1933,7 +1933,7 @@ int dvm_lbm_step(dvm_ctx *c, int nsteps, double dt, double tau)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     p.threads = dvm::lbm_threads(p.ncells, nsm);
-    p.overlap = p.ncells <= (int64_t)nsm * p.threads;
+    p.overlap = dvm::lbm_overlap(p.prec, p.ncells, nsm);
     p.status = c->d_lstatus;
     p.stream = c->stream;
     for (int s = 0; s < nsteps; s++) {

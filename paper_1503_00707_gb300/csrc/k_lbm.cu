@@ -329,11 +329,6 @@ __global__ void __launch_bounds__(256) k_lbm_moments(const T *__restrict__ f, in
 template <typename T, int DIM, int Q> int launch_t(const LbmParams &p)
 {
     const unsigned grid = (unsigned)((p.ncells + p.threads - 1) / p.threads);
-    // A step of one CTA an SM at most is bound by its launch and the codes'
-    // latency, which overlap the step before (1,388 cells D2Q9 FP64: 8.4 ->
-    // 7.0 us a step).  Larger grids hide both behind their own CTAs and keep
-    // the read-only loads (3.34M cells: 0.178 -> 0.199 ms D3Q27, 0.120 ->
-    // 0.123 D3Q19 FP32 when overlapped; 602k D3Q19: within 1%).
     if (p.overlap) {
         cudaLaunchAttribute at{};
         at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -383,6 +378,21 @@ int lbm_threads(int64_t ncells, int nsm)
     int t = 256;
     while (t > 32 && (ncells + t - 1) / t < nsm) t /= 2;
     return t;
+}
+
+// Steps that overlap the one before (their launch and the codes' latency), by
+// the cells an SM has.  FP32, at most as many as threads fit on an SM: 1.15 to
+// 1.9 times faster from 476 to 284k cells (D2Q9 5,508 cells: 4.2 -> 2.9 us;
+// D3Q19 68,880 8.3 -> 5.6, 283,640 12.2 -> 9.7), 1.07 to 1.2 at 355k; larger grids
+// hide both behind their own CTAs and keep the read-only loads (602k D3Q19
+// within 1%; 3.34M 0.120 -> 0.123 ms D3Q19, 0.178 -> 0.199 D3Q27).  FP64 is bound by
+// its pipe, and CTAs that become resident early spread unevenly over the SMs
+// once they are large (D2Q9 63,480 cells on 256 threads: 20.6 -> 28.2 us), so
+// only grids on CTAs of up to 128 threads: 1.06 to 1.36 times faster up to 20k
+// cells (D2Q9 1,388 cells: 8.3 -> 6.8 us).
+bool lbm_overlap(int prec, int64_t ncells, int nsm)
+{
+    return ncells <= (int64_t)nsm * (prec == DVM_F64 ? 128 : 2048);
 }
 
 int launch_lbm(const LbmParams &p)

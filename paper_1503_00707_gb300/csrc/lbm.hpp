@@ -53,12 +53,13 @@ struct LbmParams {
     double dt, omega;         // omega = dt / tau
     int *status;              // bit 0: a cell with rho <= 0 or non-finite moments
     int threads;              // per CTA, from lbm_threads
-    bool overlap;             // steps of one wave: each may become resident beside the one before
+    bool overlap;             // from lbm_overlap: a step may become resident beside the one before
     bool follows;             // the launch right before on the stream is a step of the same call
     cudaStream_t stream;
 };
 
 int lbm_threads(int64_t ncells, int nsm);
+bool lbm_overlap(int prec, int64_t ncells, int nsm);
 
 int launch_lbm(const LbmParams &p);
 
