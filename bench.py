@@ -432,6 +432,14 @@ def oracle_field_errors(cfg_name, prec, steps, fetch):
             "workload": cfg_name}
 
 
+def weighted_loads(b):
+    """Values that the hard-sphere sums take from one cell's f, given the
+    trials' weights: f_gamma for B, f_l and f_m for C, of the trials that carry
+    weight (the others add nothing, and the kernel does not load them)."""
+    import numpy as np
+    return 3 * int(np.count_nonzero(b))
+
+
 def hs_leg(args, name="c4_hs_bimodal"):
     """The hard-sphere collision step (Eqs. 3-6), FP32, 128 trials per node:
     on the bimodal periodic box (c4_hs_bimodal: 16,584 cells x 16^3
@@ -439,9 +447,9 @@ def hs_leg(args, name="c4_hs_bimodal"):
     253,360 cells x 24^3, Kn 0.003) from a two-beam state perturbed by up to
     5% per cell.  --hs-steps steps timed with CUDA events, then one more with
     phase events for the split between transport and the collision kernels.
-    Roofline of the collision: its shared-memory gathers, three 4-byte loads
-    per trial (f_gamma, f_l, f_m), against the derived peak of one load per
-    lane per SM clock (152 SMs x 32 lanes), over the collision phase's time
+    Roofline of the collision: its shared-memory gathers, three 4-byte values
+    per trial that carries weight (weighted_loads), against the derived peak of
+    one value per lane per SM clock (152 SMs x 32 lanes), over the collision phase's time
     (B, C and the correction; an upper bound on the gather kernel's own
     time)."""
     import numpy as np
@@ -475,8 +483,9 @@ def hs_leg(args, name="c4_hs_bimodal"):
     split, _ = s.step_timing()
     s.set_timing(False)
     nc, nv = s.ncells, s.nv
+    loads = weighted_loads(s.collision_tables(c["trials"])[3])
     s.close()
-    gathers = 3.0 * nc * nv * c["trials"]
+    gathers = float(nc) * loads
     achieved = gathers / (split[1] / 1e3)
     peak = 152 * 32 * _sm_clock_hz()
     cpu = None
@@ -509,7 +518,7 @@ def hs_leg(args, name="c4_hs_bimodal"):
         "split_ms_per_step": {"transport": split[0], "collision": split[1]},
         "roofline": {"bound": "smem", "achieved": achieved, "peak": peak, "unit": "loads/s",
                      "frac": achieved / peak, "peak_source": "derived: 152 SMs x 32 lanes x SM clock",
-                     "algorithmic_loads_per_update": 3 * c["trials"], "traffic": None},
+                     "algorithmic_loads_per_update": loads / nv, "traffic": None},
         "conservation_residual_max": _residual_ratio(resid, rs, us, Ts),
         "gpu_launches_per_step": launches / args.hs_steps, "cpu_baseline": cpu,
     }
