@@ -63,23 +63,22 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
 // k_step's partials use (total size at most 112), stay below 2^24 units, hence
 // exact in FP32, and go into 64-bit integers; the rests (of values below
 // 2^(m-30)) are summed in FP32, in at most 60 additions a value: off by less
-// than 60 2^-24 2^-54 2^m a value, 2^-60 of the warp's sum of |f| at 24^3.  The
-// warps' sums are added in FP64.  Two multiples and the rests in FP32 instead
-// (rests of 2^-30 of the cell's largest value) took 283 us where this takes 295,
-// but were up to 9.5e-13 of sum |f| off on values of that size, FP64 sums
-// 1.1e-15.  A warp with non-finite values or its largest outside [2^-71, 2^115]
-// takes FP64 sums.
+// than 60 2^-24 2^-54 2^m a value, 2^-60 of the warp's sum of |f| at 24^3, and
+// their total is rounded to u3.  The warps' sums are added in FP64.  Two
+// multiples and the rests in FP32 instead (rests of 2^-30 of the cell's largest
+// value) took 283 us where this takes 286, but were up to 9.5e-13 of sum |f| off
+// on values of that size, FP64 sums 1.1e-15.  A warp with non-finite values or
+// its largest outside [2^-71, 2^115] takes FP64 sums.
 //
 // f is read once from HBM and twice by its thread, for m and for the sums.
 // Cells of up to 56 KB go through shared memory (PIPE): a CTA takes every
 // gridDim-th cell by bulk copies, two at a time.  With SPLIT a last warp
 // finishes the cells (FP64, a long serial chain) and refills their buffers while
-// the others go on; CTAs of one or two working warps would lose a third to half
-// of an SM's warps to that and have warp 0 do it (8^3: 123 us the call, 136 with
-// it; 24^3: 399 and 371).  Larger cells are read from memory twice.  17,680
-// cells x 24^3, FP32 (0.98 GB): 4,110 us with FP64 sums, 295 us now; what bounds
-// it is the arithmetic of the split, about 800 instructions for a warp's 1,024
-// values at 54% of the issue slots.
+// the others go on (17,680 cells, calls of 16^3 184 -> 167 us, 24^3 376 -> 357);
+// a CTA of one working warp does it itself (8^3 115 us, 128 with SPLIT).  Larger
+// cells are read from memory twice.  17,680 cells x 24^3, FP32 (0.98 GB): 4,110
+// us with FP64 sums, 286 us now; what bounds it is the arithmetic of the split,
+// about 800 instructions for a warp's 1,024 values at 54% of the issue slots.
 constexpr int MOM_T = 224;
 constexpr size_t MOM_ROW = 56 * 1024;
 
@@ -246,7 +245,6 @@ __global__ void __launch_bounds__(256, 2)
     union Red {
         struct {
             int64_t hi, lo;
-            float R;
         } fx;
         double d;
     };
@@ -264,6 +262,7 @@ __global__ void __launch_bounds__(256, 2)
             bulk_g2s(tile + (size_t)b * 8 * P, f + c * 8 * (int64_t)P, bytes, &full[b]);
         }
     };
+    const double h1 = lane % 3 == 1 ? hh.x : (lane % 3 == 2 ? hh.y : hh.z), hd = lane < 4 ? h1 : h1 * h1;
     // one warp: the moments of cell c from the warps' sums
     auto finish = [&](int64_t c, int b) {
         // all are through with the cell: the one after next takes its place
@@ -273,22 +272,20 @@ __global__ void __launch_bounds__(256, 2)
         for (int w = lane < 28 ? lane / 7 : nw; w < nw; w += 4) {
             const int ex = rexp[b][w];
             const Red &r = red[b][w][k];
-            if (ex == 0) {
-                s += r.d;
-            } else {
-                const double u1 = __longlong_as_double((long long)(1023 + ex - 143) << 52);
-                s += fma((double)r.fx.hi, u1, fma((double)r.fx.lo, u1 * 0x1p-36, (double)r.fx.R));
+            double v = r.d;
+            if (ex != 0) {
+                const double u1 = __longlong_as_double((long long)(1023 + ex - 143) << 52),
+                             u3 = __longlong_as_double((long long)(1023 + ex - 179) << 52);
+                v = fma((double)r.fx.hi, u1, (double)r.fx.lo * u3);
             }
+            s = w < 4 ? v : s + v;
         }
         __syncwarp();
         if (SPLIT && lane == 0) mbar_arrive(&taken[b]);
-        s += __shfl_down_sync(0xffffffffu, s, 14);
-        s += __shfl_down_sync(0xffffffffu, s, 7);
+        if (nw > 2) s += __shfl_down_sync(0xffffffffu, s, 14);
+        if (nw > 1) s += __shfl_down_sync(0xffffffffu, s, 7);
         // lane 0: sum f; 1..3: u_d; 4..6: sum xi_d^2 f / sum f
-        const double s0 = __shfl_sync(0xffffffffu, s, 0);
-        const int d = (lane + 2) % 3;
-        const double h1 = d == 0 ? hh.x : (d == 1 ? hh.y : hh.z);
-        const double v = s / s0 * (lane < 4 ? h1 : h1 * h1);
+        const double s0 = __shfl_sync(0xffffffffu, s, 0), v = s / s0 * hd;
         const double u2 = v * v, e2 = __shfl_down_sync(0xffffffffu, v, 3);
         const double ux2 = __shfl_sync(0xffffffffu, u2, 1), uy2 = __shfl_sync(0xffffffffu, u2, 2),
                      uz2 = __shfl_sync(0xffffffffu, u2, 3);
@@ -296,8 +293,10 @@ __global__ void __launch_bounds__(256, 2)
                      ez2 = __shfl_sync(0xffffffffu, e2, 3);
         double *o = out + c * 5;
         if (lane == 0) {
+            // a third of x: the product with 1/3, corrected by its remainder (Markstein, 1990)
+            const double x = ex2 + ey2 + ez2 - (ux2 + uy2 + uz2), third = 1.0 / 3.0, t = x * third;
             o[0] = s0 * dV;
-            o[4] = (ex2 + ey2 + ez2 - (ux2 + uy2 + uz2)) / 3.0;
+            o[4] = fma(fma(-3.0, t, x), third, t);
         } else if (lane < 4) {
             o[lane] = v;
         }
@@ -385,8 +384,9 @@ __global__ void __launch_bounds__(256, 2)
         const bool mine = (lane & 3) == 0 && lane < 28;
         if (ex) {
             const int64_t hi = warp_reduce7<int64_t>(m.hi, lane), lo = warp_reduce7<int64_t>(m.lo, lane);
-            const float R = warp_reduce7<float>(m.R, lane);
-            if (mine) red[buf][warp][lane >> 2].fx = {hi, lo, R};
+            // the warp's rests, below 2^27 u3, rounded to u3
+            const float R = warp_reduce7<float>(m.R, lane) * __int_as_float((306 - ex) << 23);
+            if (mine) red[buf][warp][lane >> 2].fx = {hi, lo + __float2int_rn(R)};
         } else {
             const double t = warp_reduce7<double>(md, lane);
             if (mine) red[buf][warp][lane >> 2].d = t;
@@ -457,11 +457,12 @@ template <typename TS> int moments_t(const void *f, int64_t ncells, const MomGri
 {
     const int P = g.half[0] * g.half[1] * g.half[2], Q = P / Store<TS>::VEC;
     const TS *ft = static_cast<const TS *>(f);
-    // one quad a thread up to MOM_T quads, then two or more, evenly (24^3: 432
-    // quads on 224 threads)
-    const int rounds = (Q + MOM_T - 1) / MOM_T, t = ((Q + rounds - 1) / rounds + 31) / 32 * 32;
+    // up to two quads a thread on one warp (24 x 8 x 8 with 48 quads: 122 us the
+    // call, 137 on two warps), then one up to MOM_T quads, then two or more,
+    // evenly (24^3: 432 quads on 224 threads)
+    const int rounds = (Q + MOM_T - 1) / MOM_T, t = Q <= 64 ? 32 : ((Q + rounds - 1) / rounds + 31) / 32 * 32;
     if ((size_t)8 * P * sizeof(TS) > MOM_ROW) return moments_k<TS, false, false>(ft, ncells, g, t, out, s);
-    if (t >= 96) return moments_k<TS, true, true>(ft, ncells, g, t, out, s);
+    if (t > 32) return moments_k<TS, true, true>(ft, ncells, g, t, out, s);
     return moments_k<TS, true, false>(ft, ncells, g, t, out, s);
 }
 
