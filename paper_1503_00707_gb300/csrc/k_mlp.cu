@@ -11,14 +11,14 @@
 // the transposed copies of the forward pass; the output gradient with loss and
 // bias-gradient sums; the SiLU derivative of the backward pass.  The weight
 // gradients (C = dZ^T . activation, long K) of all four layers are one launch,
-// split over K.  Forward, backward and the Adam update all run on the device.
+// split over K up to 12,000 rows.  Forward, backward and the Adam update all run on the device.
 //
 // Bound by the latency of a few dependent chunks per launch (the network is
 // 3.1 GFLOP a pass at 24k rows): with 16-byte loads through registers, two
 // stages and 128 threads a 256 x 256 layer took 52 us on 24,032 rows, 38 us on
 // 8,192, and the weight gradients, on two CTAs each, most of a gradient's
 // 2.9 ms.  Now 14 us (24,032 rows, inference), 20 to 23 us with the transposed copies of
-// training (8,192 rows), and 15 us for all weight gradients; the whole gradient
+// training (8,192 rows), and 15 us for all their weight gradients; the whole gradient
 // takes 9 launches instead of 24.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -458,13 +458,15 @@ int mlp_cast(Mlp &m, cudaStream_t s)
 const float *mlp_bias(const Mlp &m, int l) { return m.w + param_offset(l) + (size_t)L_IN[l] * L_OUT[l]; }
 
 // K splits of the weight gradients: the seven tiles on about all 152 SMs for
-// batches up to 12,000 rows, one chain for larger ones.  The tensor core
-// truncates as it accumulates, so that a chain's sum drifts from the exact one
-// as it grows (relative to the gradient's norm: 1.8e-6 at 3,000 rows, 7e-6 at
-// 8,192, 1.8e-5 at 16,000, 8.5e-5 at 60,000); split sums are the more exact
-// ones, but beyond 12,000 rows they would move a gradient by more than 2e-5
-// from the one-chain value that earlier training runs were made with.  One chain on
-// pipelined loads takes 0.26 ms more at 30,000 rows than 21 splits.
+// batches up to 12,000 rows, one chain for larger ones.  The line is no line of
+// speed or of precision, split sums are better on either side of it: the tensor
+// core truncates as it accumulates, so that a sum drifts from the exact one with
+// the length of its chain (relative to the gradient's norm, one chain 1.1e-5 at
+// 12,008 rows, 3.4e-5 at 30,000, 7.6e-5 at 60,000; 21 splits 3e-7, 8e-7, 1.7e-6),
+// and a whole gradient takes 401, 757 and 1,380 us with one chain, 294, 479 and 850
+// with splits.  It keeps a gradient within 2e-5 of the one-chain value, which
+// gradients of every size had before there were splits, so that runs can be
+// compared with older ones to FP32 rounding.
 static int wgrad_splits(int64_t n) { return n <= 12000 ? (int)std::min<int64_t>(21, (n + 63) / 64) : 1; }
 
 // one set of working buffers for a batch of n rows (n padded to a multiple of 64)
