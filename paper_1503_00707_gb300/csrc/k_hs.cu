@@ -688,7 +688,8 @@ static int run_batches(const BcLaunch &L, const HsTables &t, float *f, float *bc
         }
         count_launch();
         // pairs of z nodes per sign group over rounds of at most CT threads,
-        // evenly (24^3: 864 on 4 x 224)
+        // evenly (24^3: 864 in 7 rounds of 124, on 128 threads)
+        static_assert(CT % 32 == 0, "the rounding below stays within k_hs_corr's part[][CT]");
         const int units = nv / 16, rounds = (units + CT - 1) / CT, per = (units + rounds - 1) / rounds;
         k_hs_corr<<<rows, (per + 31) / 32 * 32, 0, s>>>(f, Bp, Cp, t.d_xi, t.hh, c.dV, c.mom, nv,
                                                         make_int3(t.half[0], t.half[1], t.half[2]), c.dtkn, rw,

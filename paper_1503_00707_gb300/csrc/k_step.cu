@@ -110,7 +110,6 @@ template <typename TC> struct CellSlot {
                          // source for group 0, wall flip folded in
     int32_t src[24];     // per list (axis x side) up to 4 sources: cell | group flip << 28
     TC w[24];            // A_k / V_j
-    int cnt[6];
     uint32_t xmask;      // bit 4 L + k: list L has a source k >= 1
     TC invh;
 };
@@ -395,10 +394,13 @@ __device__ inline int solve_cell(const StepParams &p, StepSmem<TC> &sm, const Co
     // moments.  That solve is itself the next Newton step, with 1 + d.phi for
     // its exponential (O(d^2) apart), and Newton's steps shrink quadratically,
     // so the iteration stops when a step falls below ENT_TOL: d is then about
-    // ENT_TOL^2 and the target within 1e-11 (FP64: 1e-18) of the exponential.
-    // Iterating until a step confirmed it (1e-5, FP64 1e-9) took one more for
-    // every cell (18k cells x 24^3 FP32, stream at Mach 5: 773 -> 737 us; 8^3 to
-    // 24^3 grids in every precision: 1.15 to 1.34 times faster).
+    // ENT_TOL^2.  Against the exponential iterated to rounding, over 3,700 states
+    // on grids of 8^3 to 16^3 (T 0.15 to 6, drifts up to the grid's edge less
+    // 2.5): FP32 off by at most 2.5e-11 in norm and, at the worst node, 1.8e-8 of
+    // its value (the grid's edge, where |c|^2 multiplies d; an FP32 rounding is
+    // 6e-8); FP64 4e-15 in norm, which is rounding.  Iterating until a step
+    // confirmed it (1e-5, FP64 1e-9) took one more for every cell (18k cells x
+    // 24^3 FP32, stream at Mach 5: 773 -> 737 us).
     constexpr bool ENT = COLL == DVM_COLL_BGK_ENTROPIC;
     constexpr int NIT = ENT ? 8 : 1;
     const TC ENT_TOL = sizeof(TC) == 8 ? (TC)2e-5 : (TC)1e-3;
@@ -740,7 +742,6 @@ __global__ void __launch_bounds__(SMALL ? 192 : MAXT, SMALL ? 3 : 1) k_step(cons
                 sl.w[lane] = t.w;
             }
             if (lane < 6) {
-                sl.cnt[lane] = t.cnt;
                 // group o reads source group o ^ flip = o -/+ flip for the minus/plus list
                 const int32_t flip = t.first >> 28;
                 sl.sidx[lane] = (t.first & 0x0fffffff) * 8 + ((lane & 1) ? flip : -flip);

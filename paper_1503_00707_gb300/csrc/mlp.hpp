@@ -15,7 +15,7 @@ constexpr int64_t MLP_NPARAM = 164672;
 enum { W_X = 0, W_H, W_XT, W_Z, W_HT, W_DO, W_DOT, W_DZ, W_DZT, W_PART, W_BIAS, W_LOSS, W_R0, W_R1, MLP_NWORK };
 // what a call needs of them: the forward pass W_X and W_H, a gradient all up to
 // W_LOSS, a call on host rows W_R0 and W_R1 (with neither nor the gradient's, an
-// inference-only user holds a third of the memory)
+// inference-only user holds a sixth of the memory)
 enum { MLP_FORWARD = 0, MLP_GRAD, MLP_HOST_ROWS, MLP_NSETS };
 
 struct DevBuf {
