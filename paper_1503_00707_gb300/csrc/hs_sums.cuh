@@ -145,8 +145,7 @@ DVM_HD void add_losses(Acc2 (&acc)[NSUM], float2 (&f)[8], float2 (&B)[8], float 
         put(11, 2, b * j2);       // (j_y, |j|^2)
         put(12, 0, cz * cz);      // (j_z, j_z)
         put(13, 3, cz * j2);      // (j_z, |j|^2)
-        put(14, 0, j2 * j2);      // (|j|^2, |j|^2): the one weight that may pass 2^24 (64 x 20 x 20 nodes)
-        acc[14].e = std::fma(e ? V[0].y : V[0].x, std::fma(j2, j2, -f_mul(j2, j2)), acc[14].e);
+        put(14, 0, j2 * j2);      // (|j|^2, |j|^2): below 2^23 (at most 32 nodes an axis)
     }
 }
 

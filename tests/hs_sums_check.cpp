@@ -71,7 +71,6 @@ int main(int argc, char **argv)
                                 sum[k] += w * psi[r] * psi[s];
                                 size[k] += std::fabs((double)(w * psi[r] * psi[s]));
                                 acc2_prod(one[k], wh, wl, psi[r] * psi[s]);
-                                one[k].e += wh * std::fma(psi[r], psi[s], -(psi[r] * psi[s]));
                             }
                         for (int r = 0; r < 5; r++, k++) {
                             sum[k] += g * psi[r];

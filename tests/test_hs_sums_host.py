@@ -1,12 +1,13 @@
 """The sums of the hard-sphere correction's moment system (library code in
 paper_1503_00707_gb300/csrc/hs_sums.cuh, compiled into a small checker with
-g++) against extended precision, on cubic, small and the longest grids.
+g++) against extended precision, on cubic, small and the longest grids
+(32 nodes an axis, the most that the operator takes).
 
-A thread's Sum2 accumulation of m terms is off by at most about (m 2^-24)^2 of
-the terms' sizes, and each pair of nodes adds a rest of 2^-38 summed with
-roundings of 2^-24: 16 nodes a thread's chain of 27 pairs stay below 2^-46
-(1.4e-14), and their root mean square below 2^-49 (1.8e-15).  The sums are also
-to be no less exact than every node added by itself in Sum2."""
+A thread adds up to 28 terms to a sum, each with a rounding of 2^-48 of it (Sum2)
+and a rest of 2^-38 of its values summed with roundings of 2^-24; the threads of a
+cell average them out: below 2^-46 (1.4e-14) of the terms' sizes at most, 2^-49
+(1.8e-15) in the root mean square.  The sums are also to be no less exact than every
+node added by itself in Sum2."""
 import os
 import shutil
 import subprocess
@@ -27,9 +28,9 @@ def checker(tmp_path_factory):
     return exe
 
 
-# nodes of a sign group and threads: 4 x 4 x 8, 8^3, 14 x 16 x 16, 16^3, 24^3, 60 x 20 x 16, 64 x 50 x 8
+# nodes of a sign group and threads: 4 x 4 x 8, 8^3, 14 x 16 x 16, 16^3, 24^3, 32 x 10 x 32, 32 x 32 x 24
 @pytest.mark.parametrize("half, threads", [((2, 2, 4), 32), ((4, 4, 4), 32), ((7, 8, 8), 128), ((8, 8, 8), 128),
-                                           ((12, 12, 12), 128), ((30, 10, 8), 128), ((32, 25, 4), 128)])
+                                           ((12, 12, 12), 128), ((16, 5, 16), 128), ((16, 16, 12), 128)])
 def test_sums(checker, half, threads):
     out = subprocess.run([checker, *map(str, half), str(threads)], capture_output=True, text=True, timeout=600,
                          check=True).stdout.splitlines()
