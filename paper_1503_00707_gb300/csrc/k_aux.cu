@@ -66,9 +66,10 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
 // than 60 2^-24 2^-54 2^m a value, 2^-60 of the warp's sum of |f| at 24^3, and
 // their total is rounded to u3.  The warps' sums are added in FP64.  Two
 // multiples and the rests in FP32 instead (rests of 2^-30 of the cell's largest
-// value) took 283 us where this takes 286, but were up to 9.5e-13 of sum |f| off
+// value) took 283 us where this takes 282, but were up to 9.5e-13 of sum |f| off
 // on values of that size, FP64 sums 1.1e-15.  A warp with non-finite values or
-// its largest outside [2^-71, 2^115] takes FP64 sums.
+// its largest above 2^115 takes FP64 sums; one with its largest below 2^-71
+// scales its values by 2^96.
 //
 // f is read once from HBM and twice by its thread, for m and for the sums.
 // Cells of up to 56 KB go through shared memory (PIPE): a CTA takes every
@@ -77,9 +78,9 @@ __global__ void k_init(TS *f, int64_t ncells, int nv, int nmix, const double *w,
 // the others go on (17,680 cells, calls of 16^3 184 -> 167 us, 24^3 376 -> 357);
 // a CTA of one working warp does it itself (8^3 115 us, 128 with SPLIT).  Larger
 // cells are read from memory twice.  17,680 cells x 24^3, FP32 (0.98 GB): 4,110
-// us with FP64 sums, 286 us now; what bounds it is the arithmetic of the split,
+// us with FP64 sums, 282 us now; what bounds it is the arithmetic of the split,
 // about 800 instructions for a warp's 1,024 values at 54% of the issue slots.
-constexpr int MOM_T = 224;
+constexpr int MOM_T = 224, MOM_FP64 = 1 << 20;
 constexpr size_t MOM_ROW = 56 * 1024;
 
 // the largest of |a|, |b|, |c|, NaN if one is
@@ -231,6 +232,23 @@ template <typename TC> __device__ inline void add_quad_f64(const QV<TC> (&x)[8],
     weighted_sums<double>(s, (double)jx, (double)jy, (double)jz, m);
 }
 
+// The thread's values of a cell in shared memory times 2^96.  A call: inlined,
+// these few instructions that most warps never run slow the others (fields of
+// 17,680 cells x 24^3 727 us, 709 so).
+template <typename TS> __device__ __noinline__ void scale_tile(TS *tile, int P, int Q, int T)
+{
+    using IO = QIO<TS>;
+    constexpr int VEC = Store<TS>::VEC;
+    if constexpr (sizeof(TS) < 8) {
+        for (int q = threadIdx.x; q < Q; q += T)
+            for (int o = 0; o < 8; o++) {
+                TS *at = tile + (size_t)o * P + q * VEC;
+                IO::sts(at, q_mul(IO::lds(at), q_splat(0x1p96f)));
+            }
+        fence_proxy_async();  // before the copy that takes the place
+    }
+}
+
 // barriers of k_moments: the sums of buffer 0 or 1 are ready
 constexpr int BAR_READY = 1;
 
@@ -250,7 +268,7 @@ __global__ void __launch_bounds__(256, 2)
     };
     extern __shared__ __align__(128) unsigned char mom_tile[];  // PIPE: [2][8 P]
     __shared__ Red red[2][MOM_T / 32][7];
-    __shared__ int rexp[2][MOM_T / 32];  // exponent of the warp's largest value, 0: FP64 sums
+    __shared__ int rexp[2][MOM_T / 32];  // exponent of the warp's largest value, or MOM_FP64
     __shared__ __align__(8) uint64_t full[2], taken[2];  // the cell has arrived; its sums have been read
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x - (SPLIT ? 32 : 0), nw = T >> 5,
               Q = P / VEC;
@@ -273,7 +291,7 @@ __global__ void __launch_bounds__(256, 2)
             const int ex = rexp[b][w];
             const Red &r = red[b][w][k];
             double v = r.d;
-            if (ex != 0) {
+            if (ex != MOM_FP64) {
                 const double u1 = __longlong_as_double((long long)(1023 + ex - 143) << 52),
                              u3 = __longlong_as_double((long long)(1023 + ex - 179) << 52);
                 v = fma((double)r.fx.hi, u1, (double)r.fx.lo * u3);
@@ -341,7 +359,7 @@ __global__ void __launch_bounds__(256, 2)
             if (PIPE && q < 2 * T) return q == tid ? j0 : j1;
             return node(q);
         };
-        int ex = 0;
+        int ex = 0;  // exponent of the warp's largest value, + 256 where scaled; 0: FP64 sums
         MomSum m{};
         if constexpr (sizeof(TC) == 4) {
             float top = 0.0f;
@@ -352,15 +370,24 @@ __global__ void __launch_bounds__(256, 2)
                 for (int o = 0; o < 8; o++)
                     top = max_abs(max_abs(top, x[o].a.x, x[o].a.y), x[o].b.x, x[o].b.y);
             }
-            ex = (int)(__reduce_max_sync(0xffffffffu, __float_as_uint(top)) >> 23);
-            if (ex < 56 || ex > 240) ex = 0;
+            const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+            ex = (int)(__float_as_uint(most) >> 23);
+            if (ex < 56) {
+                // the far corner of a grid: values scaled, no FP64 sums
+                ex = 256 + max(56, (int)(__float_as_uint(most * 0x1p96f) >> 23));
+                if constexpr (PIPE) scale_tile<TS>(tile + (size_t)buf * 8 * P, P, Q, T);
+            }
+            if ((ex & 255) > 240) ex = 0;
             if (ex) {
 #pragma unroll 1
                 for (int q = tid; q < Q; q += T) {
                     QV<float> x[8];
                     load(q, x);
+                    if (!PIPE && ex >= 256)
+#pragma unroll
+                        for (int o = 0; o < 8; o++) x[o] = q_mul(x[o], q_splat(0x1p96f));
                     const int3 j = place(q);
-                    add_quad<sizeof(TS) == 2>(x, ex, j.x, j.y, j.z, m);
+                    add_quad<sizeof(TS) == 2>(x, ex & 255, j.x, j.y, j.z, m);
                 }
             }
         }
@@ -385,13 +412,13 @@ __global__ void __launch_bounds__(256, 2)
         if (ex) {
             const int64_t hi = warp_reduce7<int64_t>(m.hi, lane), lo = warp_reduce7<int64_t>(m.lo, lane);
             // the warp's rests, below 2^27 u3, rounded to u3
-            const float R = warp_reduce7<float>(m.R, lane) * __int_as_float((306 - ex) << 23);
+            const float R = warp_reduce7<float>(m.R, lane) * __int_as_float((306 - (ex & 255)) << 23);
             if (mine) red[buf][warp][lane >> 2].fx = {hi, lo + __float2int_rn(R)};
         } else {
             const double t = warp_reduce7<double>(md, lane);
             if (mine) red[buf][warp][lane >> 2].d = t;
         }
-        if (lane == 0) rexp[buf][warp] = ex;
+        if (lane == 0) rexp[buf][warp] = ex == 0 ? MOM_FP64 : ex < 256 ? ex : ex - 256 - 96;
         __syncwarp();
         if constexpr (SPLIT) {
             bar_arrive_n(BAR_READY + buf, T + 32);
@@ -458,9 +485,12 @@ template <typename TS> int moments_t(const void *f, int64_t ncells, const MomGri
     const int P = g.half[0] * g.half[1] * g.half[2], Q = P / Store<TS>::VEC;
     const TS *ft = static_cast<const TS *>(f);
     // up to two quads a thread on one warp (24 x 8 x 8 with 48 quads: 122 us the
-    // call, 137 on two warps), then one up to MOM_T quads, then two or more,
-    // evenly (24^3: 432 quads on 224 threads)
-    const int rounds = (Q + MOM_T - 1) / MOM_T, t = Q <= 64 ? 32 : ((Q + rounds - 1) / rounds + 31) / 32 * 32;
+    // call, 137 on two warps) or on three and the last one (129 to 192 quads; five
+    // or six and the last one spread unevenly over an SM's four schedulers, and two
+    // such CTAs fit it: 11,632 cells x 20 x 16 x 16 129 us, 156 on five); else one up to
+    // MOM_T quads, then two or more, evenly (24^3: 432 quads on 224 threads)
+    const int rounds = (Q + MOM_T - 1) / MOM_T, even = ((Q + rounds - 1) / rounds + 31) / 32 * 32;
+    const int t = Q <= 64 ? 32 : Q > 128 && Q <= 192 ? 96 : even;
     if ((size_t)8 * P * sizeof(TS) > MOM_ROW) return moments_k<TS, false, false>(ft, ncells, g, t, out, s);
     if (t > 32) return moments_k<TS, true, true>(ft, ncells, g, t, out, s);
     return moments_k<TS, true, false>(ft, ncells, g, t, out, s);

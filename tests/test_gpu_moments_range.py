@@ -1,6 +1,7 @@
 """Moments of a stored f whose values span many binary orders: one value of 1
 among values of `low` and below, so that the sums' second and third levels and
-their rests carry most of the values.
+their rests carry most of the values; the same scaled down, where warps without
+the large value leave the range that needs no scaling.
 
 A thread's 32 values go into integers exactly but for rests below 2^-50 of the
 largest |f|, summed in FP32 in at most 60 additions a value: off by at most
@@ -16,8 +17,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", ["f32", "bf16"])
-@pytest.mark.parametrize("n", [(6, 2, 8), (24, 24, 24), (18, 22, 32), (32, 32, 32)])
-def test_one_large_value(n, prec):
+@pytest.mark.parametrize("n", [(6, 2, 8), (18, 18, 16), (24, 24, 24), (18, 22, 32), (32, 32, 32)])
+@pytest.mark.parametrize("scale", [0, -70, -110])
+def test_one_large_value(n, prec, scale):
     s = D.Solver({"f32": D.F32, "bf16": D.BF16}[prec], D.COLL_NONE, 1.0)
     s.build_tree(D.tree_spec(3, 1, 1))
     hi = (3.0, 4.0, 5.0)
@@ -27,7 +29,7 @@ def test_one_large_value(n, prec):
     f = low[:, None] * g.uniform(0.5, 1.0, (s.ncells, s.nv))
     f[3] = 0.93 * 2.0 ** -30
     f[np.arange(8), g.integers(0, s.nv, 8)] = 1.0
-    f = storage_round(f, prec)
+    f = storage_round(f * 2.0 ** scale, prec)
     s.set_f(f)
     rho, u, T = s.moments()
     xi, dv = s.velocities().astype(np.longdouble), np.prod([2 * h / k for h, k in zip(hi, n)])
