@@ -485,12 +485,15 @@ template <typename TS> int moments_t(const void *f, int64_t ncells, const MomGri
     const int P = g.half[0] * g.half[1] * g.half[2], Q = P / Store<TS>::VEC;
     const TS *ft = static_cast<const TS *>(f);
     // up to two quads a thread on one warp (24 x 8 x 8 with 48 quads: 122 us the
-    // call, 137 on two warps) or on three and the last one (129 to 192 quads; five
-    // or six and the last one spread unevenly over an SM's four schedulers, and two
-    // such CTAs fit it: 11,632 cells x 20 x 16 x 16 129 us, 156 on five); else one up to
-    // MOM_T quads, then two or more, evenly (24^3: 432 quads on 224 threads)
+    // call, 137 on two warps); else one up to MOM_T quads, then two or more, evenly
+    // (24^3: 432 quads on 224 threads).  Five or six warps and the last one spread
+    // unevenly over an SM's four schedulers, and two such CTAs fit it: three warps
+    // take their place where shared memory holds four CTAs (11,632 cells x 20 x 16 x
+    // 16 FP32 156 -> 129 us, 20 x 20 x 24 BF16 243 -> 200; 20 x 20 x 24 FP32, where it does
+    // not, 223 -> 240).
     const int rounds = (Q + MOM_T - 1) / MOM_T, even = ((Q + rounds - 1) / rounds + 31) / 32 * 32;
-    const int t = Q <= 64 ? 32 : Q > 128 && Q <= 192 ? 96 : even;
+    const bool four = (size_t)8 * 8 * P * sizeof(TS) <= 216 * 1024;
+    const int t = Q <= 64 ? 32 : four && (even == 160 || even == 192) ? 96 : even;
     if ((size_t)8 * P * sizeof(TS) > MOM_ROW) return moments_k<TS, false, false>(ft, ncells, g, t, out, s);
     if (t > 32) return moments_k<TS, true, true>(ft, ncells, g, t, out, s);
     return moments_k<TS, true, false>(ft, ncells, g, t, out, s);
