@@ -33,7 +33,6 @@
 #include "common.cuh"
 #include "hs.hpp"
 #include "hs_sums.cuh"
-#include "quads.cuh"
 
 namespace dvm {
 
@@ -417,7 +416,7 @@ __global__ void __launch_bounds__(CT, 5)
         // al = (h/2)/sqrt(T), be = -u/sqrt(T); the system A^ e = c^ with
         // e = (1, 0, 0, 0, 0) + L^T d is factored through the well-conditioned
         // centred-basis matrix L A^ L^T (an LDL^T on lane 0) and refined
-        // against the FP64 residual of the exact sums.  The factor is FP32
+        // against the FP64 residual of the sums.  The factor is FP32
         // with four rounds (each gains at least three digits; FP64 runs at
         // 1/64 of the FP32 rate, and an FP64 factor with two rounds took a
         // third of this kernel's time at 16^3); where it does not converge
